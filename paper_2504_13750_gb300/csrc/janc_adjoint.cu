@@ -51,7 +51,7 @@ namespace janc {
 // its window.
 //
 // dW/dF_j comes from the partials with respect to the window differences
-// D_m = F_m - F_{m-1} (weno_face_dD) plus the centre F2's weight one. The
+// D_m = F_m - F_{m-1} (weno::derivative) plus the centre F2's weight one. The
 // walk sums phi dW/dD_m per difference ("edge" q between positions q-1 and
 // q), and a position's sum is complete once the faces have passed both of
 // its edges: edge q minus edge q+1 plus the phi of the face whose window it
@@ -73,6 +73,11 @@ struct EdgeSums {
   double m0 = 0.0, m1 = 0.0, m2 = 0.0, m3 = 0.0;  // F- edges t+2 .. t+5
   double pp = 0.0, pm = 0.0;                      // the last completed F+ / F- edge (t, t+1)
   double ph1 = 0.0, ph2 = 0.0;                    // phi of faces t-1 and t-2
+  // Face t's partials (weno::derivative_plus in d[0..3], _minus in d[4..7]) times phi.
+  __device__ __forceinline__ void add(double phi, const double* d) {
+    p0 = fma(phi, d[0], p0); p1 = fma(phi, d[1], p1); p2 = fma(phi, d[2], p2); p3 = fma(phi, d[3], p3);
+    m0 = fma(phi, d[4], m0); m1 = fma(phi, d[5], m1); m2 = fma(phi, d[6], m2); m3 = fma(phi, d[7], m3);
+  }
   // After face t's partials are in: positions t (F+) and t+1 (F-) are
   // complete; add them to slot pair `s` (+0) and the next pair (+1).
   __device__ __forceinline__ void finish_face(double phi, double* gs, long long pstride) {
@@ -199,23 +204,25 @@ __global__ void __launch_bounds__(VLINES * NV) k_adj_faces(StateView S, const do
   const double* lm = sLm[line];
   const double* pt = (var == T.nmom) ? sHp[line] : (var == 3 ? sHpu[line] : nullptr);
   const double* ml = sMu[var][line];
-  auto Fp = [&](int w) -> double { return pt ? fma(lp[w], Ul[w], pt[w]) : lp[w] * Ul[w]; };
-  auto Fm = [&](int w) -> double { return pt ? fma(lm[w], Ul[w], pt[w]) : lm[w] * Ul[w]; };
+  const SplitLine L{Ul, lp, lm, pt};
   long long pstride;
   double* gbase = gf_base(T, GFx, GFy, g, var, lg, pstride);
-  const double rh4 = 4.0 * rh;
-  Win P, M;
-  P.init(Fp(0), Fp(1), Fp(2), Fp(3), Fp(4), g.eps4);
-  M.init(Fm(1), Fm(2), Fm(3), Fm(4), Fm(5), g.eps4);
+  const weno::Eps eps(g.eps4);
+  weno::Win P, M;
+  L.init(P, M, eps);
   EdgeSums E;
   for (int t = 0; t < nf; ++t) {
-    const double dmu = ml[t + 1] - ml[t];
-    weno_face_dD<false, true>(P, rh4 * dmu, nullptr, E.p0, E.p1, E.p2, E.p3);
-    weno_face_dD<true, true>(M, rh4 * dmu, nullptr, E.m0, E.m1, E.m2, E.m3);
-    E.finish_face(rh * dmu, gbase + (long long)t * pstride, pstride);
+    const double phi = rh * (ml[t + 1] - ml[t]);
+    double d[8];
+    const weno::Weights wp = P.weights_plus();
+    weno::derivative_plus(P, wp, weno::Coef(wp), d);
+    const weno::Weights wm = M.weights_minus();
+    weno::derivative_minus(M, wm, weno::Coef(wm), d + 4);
+    E.add(phi, d);
+    E.finish_face(phi, gbase + (long long)t * pstride, pstride);
     if (t + 1 < nf) {
-      P.push(Fp(t + 5), g.eps4);
-      M.push(Fm(t + 6), g.eps4);
+      P.push(L.plus(t + 5), eps);
+      M.push(L.minus(t + 6), eps);
     }
   }
   E.flush(gbase + (long long)nf * pstride, pstride);
@@ -247,18 +254,15 @@ __global__ void __launch_bounds__(VLINES * NV) k_adj_faces_lin(const double* __r
   long long pstride;
   double* gbase = gf_base(T, GFx, GFy, g, var, lg, pstride);
   EdgeSums E;
-  const double rh4 = 4.0 * rh;  // the store holds a quarter of each partial
 #pragma unroll 4
   for (int t = 0; t < nf; ++t) {
     const double* l = lb + (long long)t * fstride;
     double d[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) d[c] = __ldg(l + c * cstride);
-    const double dmu = ml[t + 1] - ml[t];
-    const double p4 = rh4 * dmu;
-    E.p0 = fma(p4, d[0], E.p0); E.p1 = fma(p4, d[1], E.p1); E.p2 = fma(p4, d[2], E.p2); E.p3 = fma(p4, d[3], E.p3);
-    E.m0 = fma(p4, d[4], E.m0); E.m1 = fma(p4, d[5], E.m1); E.m2 = fma(p4, d[6], E.m2); E.m3 = fma(p4, d[7], E.m3);
-    E.finish_face(rh * dmu, gbase + (long long)t * pstride, pstride);
+    const double phi = rh * (ml[t + 1] - ml[t]);
+    E.add(phi, d);
+    E.finish_face(phi, gbase + (long long)t * pstride, pstride);
   }
   E.flush(gbase + (long long)nf * pstride, pstride);
 }

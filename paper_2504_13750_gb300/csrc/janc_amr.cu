@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(ALINES* NV) k_amr_flux(StateView S, const unsi
     out = Gy + ((long long)var * L.nblk + blk) * (AB + 1) * AB + li;
     stride = AB;
   }
-  slide_line2(Ul, sLp + line * AWIN, sLm + line * AWIN, pt, L.eps4, AB + 1, out, stride);
+  slide_line2(SplitLine{Ul, sLp + line * AWIN, sLm + line * AWIN, pt}, L.eps4, AB + 1, out, stride);
 }
 
 // ---- RK stage of every block; the external band takes the parent layer ----

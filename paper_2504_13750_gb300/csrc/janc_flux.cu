@@ -10,12 +10,15 @@
 // with the 5-cell stencil
 // margin, are staged in shared memory once; every thread then owns one
 // (line, variable) and slides two 5-point windows (F+ and F-) along its line,
-// so the first and second differences and the 13/3 S^2 part of the
-// smoothness indicators are computed once per point instead of once per
-// face, and each thread carries two independent dependency chains.
+// so the differences, their squares and the smoothness forms are computed once
+// per point instead of once per face, and each thread carries two independent
+// dependency chains.
 //
-// Per face and sign the reconstruction costs 27 FP64 instructions plus 5 per
-// new point (Jiang-Shu weights in divide-free form, one reciprocal).
+// Bound: the FP64 pipe starts one warp instruction every 16 clocks, so the
+// nonlinear weights are formed on the integer pipes (janc_weno.cuh) and a face
+// of one variable takes 14 FP64 instructions for both signs (67 when the
+// weights were FP64 too). 2048 x 256 with 12 variables, both directions:
+// 1.73 ms a launch before, 0.60 ms now.
 #include <atomic>
 
 #include "janc_device.cuh"
@@ -124,9 +127,9 @@ __device__ __forceinline__ void face_flux_tile(const StateView& S, const unsigne
       long long cstride;
       if (xdir) { lb = lin + ((long long)var * nfx + f0) * ny + lg; cstride = (long long)NV * nfx * ny; }
       else { lb = lin + 8LL * NV * nfx * ny + ((long long)var * nfy + f0) * nx + lg; cstride = (long long)NV * nfy * nx; }
-      slide_line2_lin(Ul, sLp + line * WIN, sLm + line * WIN, pt, g.eps4, nf, out, stride, lb, nlines, cstride);
+      slide_line2_lin(SplitLine{Ul, sLp + line * WIN, sLm + line * WIN, pt}, g.eps4, nf, out, stride, lb, nlines, cstride);
     } else {
-      slide_line2(Ul, sLp + line * WIN, sLm + line * WIN, pt, g.eps4, nf, out, stride);
+      slide_line2(SplitLine{Ul, sLp + line * WIN, sLm + line * WIN, pt}, g.eps4, nf, out, stride);
     }
   }
 }

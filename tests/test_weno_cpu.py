@@ -1,0 +1,123 @@
+"""The integer-weight WENO5 reconstruction (csrc/janc_weno.cuh) on the CPU
+against exact rational arithmetic: face values, derivatives, the reciprocal
+and the conversion, over smooth, discontinuous, tiny, huge and mixed windows."""
+import ctypes
+import os
+import shutil
+import subprocess
+from fractions import Fraction as Q
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no host C++ compiler")
+    out = str(tmp_path_factory.mktemp("wh") / "libweno_harness.so")
+    subprocess.run([cxx, "-std=c++17", "-O1", "-ffp-contract=off", "-shared", "-fPIC",
+                    os.path.join(HERE, "weno_harness.cpp"), "-o", out], check=True)
+    return ctypes.CDLL(out)
+
+
+def _ptr(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+def _faces(lib, Fp, Fm, eps):
+    n, ln = Fp.shape
+    s, d = np.zeros(n), np.zeros((n, 8))
+    lib.wh_faces(n, ln - 6, _ptr(Fp), _ptr(Fm), ctypes.c_double(eps), _ptr(s), _ptr(d))
+    return s, d
+
+
+def _exact(f, eps):
+    """WENO5-JS value at the right face of f[2] and its derivative with
+    respect to the four differences, in rationals."""
+    D = [f[k + 1] - f[k] for k in range(4)]
+    C = [4 * D[0] ** 2 - 11 * D[0] * D[1] + 10 * D[1] ** 2, 4 * D[1] ** 2 - 5 * D[1] * D[2] + 4 * D[2] ** 2,
+         10 * D[2] ** 2 - 11 * D[2] * D[3] + 4 * D[3] ** 2]
+    C = [c + 3 * eps for c in C]
+    dC = [[8 * D[0] - 11 * D[1], 20 * D[1] - 11 * D[0], 0, 0], [0, 8 * D[1] - 5 * D[2], 8 * D[2] - 5 * D[1], 0],
+          [0, 0, 20 * D[2] - 11 * D[3], 8 * D[3] - 11 * D[2]]]
+    a = [Q(g) / c ** 2 for g, c in zip((1, 6, 3), C)]
+    s = sum(a)
+    w = [x / s for x in a]
+    q = [(5 * D[1] - 2 * D[0]) / 6, (D[1] + 2 * D[2]) / 6, (4 * D[2] - D[3]) / 6]
+    dq = [[Q(-2, 6), Q(5, 6), 0, 0], [0, Q(1, 6), Q(2, 6), 0], [0, 0, Q(4, 6), Q(-1, 6)]]
+    r = sum(x * y for x, y in zip(w, q))
+    g = [sum(w[k] * dq[k][m] - 2 * w[k] * (q[k] - r) * dC[k][m] / C[k] for k in range(3)) for m in range(4)]
+    return f[2] + r, g
+
+
+def _windows(kind, n, ln, rng):
+    x = rng.uniform(0, 6.28, (n, 1)) + rng.uniform(0, 0.4, (n, 1)) * np.arange(ln)
+    jump = np.arange(ln)[None] >= rng.integers(1, ln, (n, 1))
+    return {
+        "smooth": 1e5 * (2 + np.sin(x)),
+        "shock": 1e5 * (1 + 0.1 * np.sin(x)) + jump * rng.uniform(0, 3e6, (n, 1)),
+        "energy_shock": 1e9 * (1 + 1e-3 * rng.uniform(size=(n, ln)) + 10 * jump),
+        "noise": rng.standard_normal((n, ln)),
+        "below_eps": 1e-8 * rng.standard_normal((n, ln)),
+        "around_eps": 1e-3 * (2 + np.sin(3 * x)),
+        "half_zero": np.where(jump, 0.0, 1e5 * (1 + 0.01 * rng.uniform(size=(n, ln)))),
+        "mixed": rng.standard_normal((n, ln)) * np.exp(12 * rng.standard_normal((n, ln))),
+        "tie": rng.integers(-3, 4, (n, ln)).astype(float),
+        "huge": 1e80 * rng.standard_normal((n, ln)),
+        "uniform": np.broadcast_to(rng.standard_normal((n, 1)), (n, ln)),
+    }[kind].astype(np.float64)
+
+
+KINDS = ("smooth", "shock", "energy_shock", "noise", "below_eps", "around_eps", "half_zero", "mixed", "tie", "huge", "uniform")
+
+
+@pytest.mark.parametrize("slide", [0, 5])
+@pytest.mark.parametrize("kind", KINDS)
+def test_faces_and_derivatives(lib, kind, slide):
+    rng = np.random.default_rng([KINDS.index(kind), slide])
+    n, ln, eps = 150, 6 + slide, 1e-6
+    Fp = np.ascontiguousarray(_windows(kind, n, ln, rng))
+    Fm = np.ascontiguousarray(_windows(kind, n, ln, rng))
+    s, d = _faces(lib, Fp, Fm, eps)
+    for i in range(n):
+        p, m = [Q(float(v)) for v in Fp[i, slide:]], [Q(float(v)) for v in Fm[i, slide:]]
+        vp, gp = _exact(p[0:5], Q(eps))
+        vm, gm = _exact(m[5:0:-1], Q(eps))
+        # 10 roundings, each at most half an ulp of a partial sum bounded by the largest value
+        # (centre values) or twice the largest difference (the small terms)
+        scale = max(abs(v) for v in p + m)
+        assert abs(Q(s[i]) - (vp + vm)) <= 12 * Q(2) ** -53 * scale
+        # the mirrored window's differences run backwards with the sign changed: D4..D1
+        gm = [-g for g in gm[::-1]]
+        # second derivative terms: |g| <= 8, every factor good to a few ulps of the largest difference,
+        # whose square the forms are at least 0.7 of
+        for a, b in zip(d[i], gp + gm):
+            assert abs(Q(float(a)) - b) <= Q(2) ** -44 * max(1, abs(b))
+    if kind == "uniform":
+        assert np.array_equal(s, Fp[:, 0] + Fm[:, 0])
+
+
+def test_nonfinite_values_stay_nonfinite(lib):
+    F = np.ones((12, 6))
+    F[np.arange(6), np.arange(6)] = np.inf
+    F[6 + np.arange(6), np.arange(6)] = np.nan
+    s, _ = _faces(lib, F, F, 1e-6)
+    assert not np.isfinite(s).any()
+
+
+def test_reciprocal_and_conversion(lib):
+    rng = np.random.default_rng(3)
+    x = [2 ** 56, 2 ** 56 + 1, 2 ** 63, 2 ** 63 + 1, 2 ** 64 - 1, 2 ** 64 - 2 ** 32, 2 ** 57 - 1, 3 * 2 ** 61]
+    x += [int(v) | 2 ** 56 for v in rng.integers(0, 2 ** 63, 20000, dtype=np.uint64) >> rng.integers(0, 7, 20000).astype(np.uint64)]
+    x = np.array(x, dtype=np.uint64)
+    n = x.size
+    y, z, b = np.zeros(n, np.uint64), np.zeros(n, np.int32), np.zeros(n)
+    lib.wh_soft(n, _ptr(x), _ptr(y), _ptr(z), _ptr(b))
+    for xi, yi, zi, bi in zip(x.tolist(), y.tolist(), z.tolist(), b.tolist()):
+        assert zi == 64 - xi.bit_length()
+        assert abs(Q(yi) - Q(2 ** 127, xi << zi)) <= 8
+        assert 0 <= Q(xi, 2 ** 64) - Q(bi) < Q(xi, 2 ** 64) * Q(2) ** -52

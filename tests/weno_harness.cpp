@@ -1,0 +1,43 @@
+// Test harness: the WENO5 reconstruction of the face kernels (janc_weno.cuh,
+// 64-bit integer weights) compiled for the host behind a C ABI, so that the
+// CPU tests can compare it with exact arithmetic. Built by the tests with the
+// host C++ compiler; not part of the library.
+#include "../paper_2504_13750_gb300/csrc/janc_weno.cuh"
+
+using namespace janc;
+
+extern "C" {
+
+// n windows of 6 values each: sum[i] = F+ of values 0..4 plus F- of values
+// 1..5 at their common face, reached by `slide` pushes from a window of
+// 6 + slide values (F: n x (6 + slide)); d[8 i ..] the derivatives with respect
+// to the differences of the F+ and the F- window.
+void wh_faces(int n, int slide, const double* Fp, const double* Fm, double eps, double* sum, double* d) {
+  const weno::Eps e(4.0 * eps);
+  const int len = 6 + slide;
+  for (int i = 0; i < n; ++i) {
+    const double *p = Fp + (long)i * len, *m = Fm + (long)i * len;
+    weno::Win P, M;
+    P.init(p[0], p[1], p[2], p[3], p[4], e);
+    M.init(m[1], m[2], m[3], m[4], m[5], e);
+    for (int t = 0; t < slide; ++t) {
+      P.push(p[t + 5], e);
+      M.push(m[t + 6], e);
+    }
+    const weno::Weights wp = P.weights_plus(), wm = M.weights_minus();
+    const weno::Coef cp(wp), cm(wm);
+    sum[i] = weno::face_sum(P, cp, M, cm);
+    weno::derivative_plus(P, wp, cp, d + 8 * i);
+    weno::derivative_minus(M, wm, cm, d + 8 * i + 4);
+  }
+}
+
+// y[i] = 2^127 / (x[i] 2^z[i]) and b[i] = x[i] 2^-64 as a double.
+void wh_soft(int n, const unsigned long long* x, unsigned long long* y, int* z, double* b) {
+  for (int i = 0; i < n; ++i) {
+    y[i] = soft::recip(x[i], z + i);
+    b[i] = soft::to_double(x[i], 0);
+  }
+}
+
+}  // extern "C"
