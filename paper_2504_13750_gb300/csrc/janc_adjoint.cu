@@ -421,7 +421,7 @@ __device__ __forceinline__ void src_grad(const double* u, double T, const MechDe
   const double rT = rcp(T);
   const double rT2 = rT * rT;
   // with `keep` the forward's k_f and k_b are read back and exp(G_k) is not needed
-  const double lnT = keep ? 0.0 : log(T);
+  const double lnT = keep ? 0.0 : log_t(T);
   double eG[NS], reG[NS], dG[NS];
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
@@ -876,7 +876,7 @@ __device__ void chem_vjp_rev(const double* u, double T, const MechDev& m, double
   double Ctot = X[0];
 #pragma unroll
   for (int k = 1; k < NS; ++k) Ctot += X[k];
-  const double lnT = log(T);
+  const double lnT = log_t(T);
   const double rT = rcp(T);
   const double rT2 = rT * rT;
   double eG[NS], reG[NS], dG[NS];

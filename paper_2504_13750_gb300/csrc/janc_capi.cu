@@ -120,6 +120,29 @@ int build_mech(const janc_mechanism* m, MechDev* h) {
     h->Wd[k] = h->invM[k] - h->WN;
     for (int q = 0; q < 6; ++q) h->hcd[k][q] = h->hc[k][q] * h->invM[k] - h->hcN[q];
   }
+  // the integer form of the mixture sums (MechDev::mixn)
+  h->mix_ok = 1;
+  for (int k = 1; k < ns; ++k) h->mixp[k] = (int)std::lround(std::log2(h->invM[k - 1] / h->WN));
+  for (int q = 0; q < 7; ++q) {
+    double c[MAX_NS];
+    int top = 0;
+    bool any = false;
+    for (int k = 0; k < ns; ++k) {
+      c[k] = q == 0 ? (k ? h->Wd[k - 1] : h->WN) : (k ? h->hcd[k - 1][q - 1] : h->hcN[q - 1]);
+      c[k] = std::ldexp(c[k], -h->mixp[k]);
+      int e;
+      std::frexp(c[k], &e);
+      if (c[k] != 0.0 && (!any || e > top)) top = e, any = true;
+    }
+    h->mixe[q] = top;
+    if (top < -400 || top > 400) h->mix_ok = 0;
+    for (int k = 0; k < ns; ++k) {
+      const double n = std::ldexp(std::fabs(c[k]), 64 - top);  // < 2^64
+      if (!(n < 0x1p64)) h->mix_ok = 0;
+      h->mixn[q][k] = n < 0x1p64 ? (unsigned long long)n : 0ull;
+      h->mixs[q][k] = c[k] < 0.0 ? 0xffffffffu : 0u;
+    }
+  }
   for (int i = 0; i < m->nr; ++i) {
     if (!(m->A[i] > 0.0)) return fail(JANC_E_INVALID, "Arrhenius A must be > 0");
     h->lnA[i] = std::log(m->A[i]);

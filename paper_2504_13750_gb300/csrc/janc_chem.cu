@@ -79,7 +79,7 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
 #pragma unroll
     for (int k = 1; k < NS; ++k) Ctot += X[k];
 
-    const double lnT = log(T);
+    const double lnT = log_t(T);
     const double rT = rcp(T);
     // exp(G_k) and exp(-G_k), G_k = s_k/R - h_k/(RT) (Eq. 4.9 bracket)
     double eG[NS], reG[NS];

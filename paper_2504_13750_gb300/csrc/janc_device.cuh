@@ -7,11 +7,14 @@
 // done exactly outside the FP64 pipe is done there: maxima of non-negative
 // doubles compare their bit patterns as integers, absolute values clear the
 // sign bit, pivot searches and row swaps are integer compares and selects,
-// and the reciprocal starts from the MUFU approximation.
+// and reciprocals, exponentials, logarithms, square roots and the mixture sums
+// are formed on 64-bit integers (janc_soft.cuh).
 #pragma once
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include "janc_soft.cuh"
 
 namespace janc {
 
@@ -65,6 +68,15 @@ struct MechDev {
   double hcd[MAX_NS][6];
   double WN;
   double Wd[MAX_NS];
+  // The same sums on integers: row 0 is W, row 1 + q coefficient q; entry 0
+  // multiplies rho, entry 1 + k rho Y_k. A coefficient is +-n 2^(mixe - 64)
+  // 2^mixp (mixs: the sign as a mask); 2^mixp is 1/M_k over 1/M_ns to a power
+  // of two, moved over to the variable so that a light species' large
+  // coefficients do not cost the others their low bits.
+  unsigned long long mixn[7][MAX_NS];
+  unsigned mixs[7][MAX_NS];
+  int mixe[7], mixp[MAX_NS];
+  int mix_ok;  // every mixe within +-400
 };
 
 // Grid constants passed by value to every kernel.
@@ -128,67 +140,28 @@ __device__ __forceinline__ bool finite_bits(double x) {
   return ((dbits(x) >> 52) & 0x7ff) != 0x7ff;
 }
 
-// Reciprocal of a normal double: the MUFU approximation (relative error
-// below 2^-20) refined by one third-order step of the iteration for 1/d,
-// x' = x (1 + e + e^2) with e = 1 - d x, which cubes the relative error
-// (2^-60, below double rounding) in three FMAs.
-__device__ __forceinline__ double rcp(double d) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  const double e = fma(-d, r, 1.0);
-  const double e2 = fma(e, e, e);
-  return fma(r, e2, r);
+// x > 0 (false for NaN), on the bits.
+__device__ __forceinline__ bool positive_bits(double x) {
+  return dbits(x) - 1ull < 0x7ff0000000000000ull;
 }
 
-// 2^(j/64), j = 0..63, rounded to double (computed to 200 bits).
-static __device__ const double kExp2Tab[64] = {
-    0x1.0000000000000p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0, 0x1.0874518759bc8p+0,
-    0x1.0b5586cf9890fp+0, 0x1.0e3ec32d3d1a2p+0, 0x1.11301d0125b51p+0, 0x1.1429aaea92de0p+0,
-    0x1.172b83c7d517bp+0, 0x1.1a35beb6fcb75p+0, 0x1.1d4873168b9aap+0, 0x1.2063b88628cd6p+0,
-    0x1.2387a6e756238p+0, 0x1.26b4565e27cddp+0, 0x1.29e9df51fdee1p+0, 0x1.2d285a6e4030bp+0,
-    0x1.306fe0a31b715p+0, 0x1.33c08b26416ffp+0, 0x1.371a7373aa9cbp+0, 0x1.3a7db34e59ff7p+0,
-    0x1.3dea64c123422p+0, 0x1.4160a21f72e2ap+0, 0x1.44e086061892dp+0, 0x1.486a2b5c13cd0p+0,
-    0x1.4bfdad5362a27p+0, 0x1.4f9b2769d2ca7p+0, 0x1.5342b569d4f82p+0, 0x1.56f4736b527dap+0,
-    0x1.5ab07dd485429p+0, 0x1.5e76f15ad2148p+0, 0x1.6247eb03a5585p+0, 0x1.6623882552225p+0,
-    0x1.6a09e667f3bcdp+0, 0x1.6dfb23c651a2fp+0, 0x1.71f75e8ec5f74p+0, 0x1.75feb564267c9p+0,
-    0x1.7a11473eb0187p+0, 0x1.7e2f336cf4e62p+0, 0x1.82589994cce13p+0, 0x1.868d99b4492edp+0,
-    0x1.8ace5422aa0dbp+0, 0x1.8f1ae99157736p+0, 0x1.93737b0cdc5e5p+0, 0x1.97d829fde4e50p+0,
-    0x1.9c49182a3f090p+0, 0x1.a0c667b5de565p+0, 0x1.a5503b23e255dp+0, 0x1.a9e6b5579fdbfp+0,
-    0x1.ae89f995ad3adp+0, 0x1.b33a2b84f15fbp+0, 0x1.b7f76f2fb5e47p+0, 0x1.bcc1e904bc1d2p+0,
-    0x1.c199bdd85529cp+0, 0x1.c67f12e57d14bp+0, 0x1.cb720dcef9069p+0, 0x1.d072d4a07897cp+0,
-    0x1.d5818dcfba487p+0, 0x1.da9e603db3285p+0, 0x1.dfc97337b9b5fp+0, 0x1.e502ee78b3ff6p+0,
-    0x1.ea4afa2a490dap+0, 0x1.efa1bee615a27p+0, 0x1.f50765b6e4540p+0, 0x1.fa7c1819e90d8p+0};
+// Reciprocal, exponential and logarithm on integers (janc_soft.cuh). As FP64
+// sequences they were 3, 10 and about 25 FP64 instructions (16 clocks each),
+// here 30, 70 and 75 instructions of which the SM starts four a clock.
+__device__ __forceinline__ double rcp(double d) { return soft::rcp_double(d); }
 
-// FP64 exponential by P. T. P. Tang's table-driven method (ACM TOMS 15(2),
-// 1989): x = (64 m + j) ln2/64 + r with |r| <= ln2/128, the reduction split
-// Cody-Waite style (L1 carries 32 significant bits, so n L1 is exact),
-// exp(r) - 1 from its Taylor series through r^5/120 (truncation below
-// 4e-17), then 2^(j/64) from the table and 2^m added to the exponent field
-// with integer instructions. 10 FP64 instructions; about 1 ulp. Results that
-// would overflow give +inf, underflow gives 0, NaN stays NaN.
+// e^x; results that would overflow give +inf, results below the normal range
+// 0, NaN stays NaN.
 __device__ __forceinline__ double exp_t(double x) {
-  constexpr double kInv = 0x1.71547652b82fep+6;  // 64 / ln 2
-  constexpr double kL1 = 0x1.62e42fee00000p-7;   // ln 2 / 64, leading part
-  constexpr double kL2 = 0x1.a39ef35793c76p-39;  // ln 2 / 64 - kL1
-  constexpr double kMagic = 0x1.8p52;            // rounds to an integer in the low mantissa bits
-  const double t = fma(x, kInv, kMagic);
-  const int n = __double2loint(t);
-  const double nd = t - kMagic;
-  double r = fma(nd, -kL1, x);
-  r = fma(nd, -kL2, r);
-  double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
-  q = fma(r, q, 1.0 / 6.0);
-  q = fma(r, q, 0.5);
-  const double p = fma(r * r, q, r);
-  const double T = __ldg(&kExp2Tab[n & 63]);
-  const double y = fma(T, p, T);
-  const int m = n >> 6;
-  double out = bitsd(dbits(y) + ((unsigned long long)(long long)m << 52));
-  const unsigned xe = (unsigned)(dbits(x) >> 52) & 0x7ffu;
-  if (m > 1023) out = bitsd(0x7ff0000000000000ull);
-  if (m < -1021) out = 0.0;
-  if (xe == 0x7ffu) out = (dbits(x) & 0xfffffffffffffull) ? x : ((long long)dbits(x) < 0 ? 0.0 : x);
-  return out;
+  if ((__double2hiint(x) & 0x7fffffff) < 0x40862000) return soft::exp_double(x);  // |x| < 708
+  const double r = exp(x);
+  return r < 0x1p-1022 ? 0.0 : r;
+}
+
+__device__ __forceinline__ double log_t(double x) {
+  const int h = __double2hiint(x);
+  if (h >= 0x40000000 && h < 0x7fd00000) return soft::log_double(x);  // [2, 2^1022)
+  return log(x);
 }
 
 // dt of the step from the alpha slot of its starting state (cfl() of Sec. 4.3).
@@ -201,9 +174,49 @@ __device__ __forceinline__ double step_dt(const StepCtl& c, const unsigned long 
 
 // W = sum_k z_k and the first NH mixture enthalpy coefficients
 // h[q] = sum_k z_k hc_k[q] (z_k = rho Y_k / M_k) from the carried variables,
-// through the folded tables of MechDev: 1 + (ns - 1) FP64 operations each.
+// through the folded tables of MechDev. On integers: the variables aligned to
+// the largest one, 62 bits each, products kept to their upper halves; an
+// error of 2^-58 of the largest term of a sum, with ns terms about 10
+// instructions each (an FP64 term is one, but of 16 clocks). Variables that
+// are not finite, extreme (beyond about 2^+-500), or whose sizes add up to more
+// than a word holds, take the FP64 sums.
 template <int NS, int NH>
 __device__ __forceinline__ void mixture_sums(const double* u, const MechDev& m, double& W, double* h) {
+  using namespace soft;
+  if (NS > 1) {
+    u64 x[NS];
+    unsigned neg[NS];
+    int e[NS], E = 0;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      const Parts p(k ? u[3 + k] : u[0]);
+      x[k] = p.m;
+      neg[k] = p.neg ? 0xffffffffu : 0u;
+      e[k] = p.e + (k ? m.mixp[k] : 0);
+      E = e[k] > E ? e[k] : E;
+    }
+    unsigned total = 0;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      x[k] = shr(x[k], E - e[k] + 2);
+      total += hi32(x[k]) >> 3;
+    }
+    if (m.mix_ok && E >= 512 && E < 1536 && total < (1u << 28) - NS) {
+#pragma unroll
+      for (int q = 0; q <= NH; ++q) {
+        u64 s = 0;
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+          const unsigned f = neg[k] ^ m.mixs[q][k];
+          const u64 t = mulhi(x[k], m.mixn[q][k]);
+          s += (t ^ (((u64)f << 32) | f)) + (f & 1u);
+        }
+        const double v = signed_double((long long)s, E - 1084 + m.mixe[q]);
+        if (q == 0) W = v; else h[q - 1] = v;
+      }
+      return;
+    }
+  }
   const double rho = u[0];
   W = rho * m.WN;
 #pragma unroll
@@ -217,6 +230,24 @@ __device__ __forceinline__ void mixture_sums(const double* u, const MechDev& m, 
   }
 }
 
+// sqrt(a b r / d), r a reciprocal: on integers for positive normal factors.
+__device__ __forceinline__ double speed(double a, double b, double r, double d) {
+  using namespace soft;
+  const Parts pa(a), pb(b), pr(r), pd(d);
+  const int lo = min(min(pa.e, pb.e), min(pr.e, pd.e)), hi = max(max(pa.e, pb.e), max(pr.e, pd.e));
+  if (lo >= 512 && hi < 1536 && !(pa.neg | pb.neg | pr.neg | pd.neg)) {
+    // a b r / d = n 2^(e - 64) with e even and n in [2^62, 2^64)
+    const u64 t = mulhi(mulhi(pa.m, pb.m), mulhi(pr.m, recip_normal(pd.m)));
+    int e = pa.e + pb.e + pr.e - 1086 * 3 + 959 - pd.e + 64 * 3 + 64;
+    const Num n = normal(t, e);
+    e = n.e;
+    const u64 s = sqrt_q((e & 1) ? n.n >> 1 : n.n);  // in [2^63, 2^64)
+    e += e & 1;
+    return round_double(s, e / 2 - 1);
+  }
+  return sqrt(a * b * r * rcp(d));
+}
+
 // Sound speed exactly as newton_cell finishes it, from the stored T.
 template <int NS>
 __device__ __forceinline__ double sound_speed(const double* u, double t, const MechDev& m) {
@@ -228,7 +259,7 @@ __device__ __forceinline__ double sound_speed(const double* u, double t, const M
   const double Cv = fma(t, fma(t, fma(t, fma(t, c4, c3), c2), c1), K1);
   const double Cp = Cv + W;
   const double p = RU * W * t;
-  return sqrt(Cp * p * rrho * rcp(Cv));
+  return speed(Cp, p, rrho, Cv);
 }
 
 // Molar production rates (Eq. 4.7-4.9) of the carried species k < ns - 1 at
@@ -252,7 +283,7 @@ __device__ __forceinline__ void carried_rates(const double* u, double T, const M
   double Ctot = X[0];
 #pragma unroll
   for (int k = 1; k < NS; ++k) Ctot += X[k];
-  const double lnT = log(T);
+  const double lnT = log_t(T);
   const double rT = rcp(T);
   double eG[NS], reG[NS];
 #pragma unroll
@@ -372,7 +403,9 @@ __device__ __forceinline__ void block_reduce_alpha_status(unsigned long long sx,
 //   H(T) = sum_k z_k h_k(T)/Ru with z_k = rho Y_k / M_k,
 //   F(T) = H(T) - W T - rho e / Ru  (W = sum_k z_k, rho e = E - |rho u|^2 / (2 rho)),
 //   F'(T) = sum_k z_k cv_k / Ru.
-// Stops when |dT| <= tol * T after the update. Returns status bits.
+// Stops when |dT| <= tol * T after the update, or, with another iteration
+// allowed to confirm it, at |dT| <= 2^-28 T: the next correction would be
+// below T dT^2 F''/2F' < 2^-54 T. Returns status bits.
 template <int NS>
 __device__ __forceinline__ int newton_cell(const double* u, double Tw, const MechDev& m, double tol, int maxit,
                                            double& T, double& p, double& c, double& rrho) {
@@ -385,6 +418,7 @@ __device__ __forceinline__ int newton_cell(const double* u, double Tw, const Mec
   const double rhoe_R = fma(-0.5 * rrho, ke, u[3]) * (1.0 / RU);
   const double K0 = h[5] - rhoe_R;
   const double K1 = h[0] - W;
+  const bool early = tol >= 0x1p-50 && tol <= 0x1p-28;
   double t = Tw;
   int st = 0;
   int it = 0;
@@ -393,15 +427,19 @@ __device__ __forceinline__ int newton_cell(const double* u, double Tw, const Mec
     double Fp = fma(t, fma(t, fma(t, fma(t, c4, c3), c2), c1), K1);
     double dT = -F * rcp(Fp);
     t += dT;
-    if (!(dabs(dT) > tol * dabs(t))) break;
+    // the early test on integers: 2^28 |dT| by its exponent field
+    const bool done = early && it + 1 < maxit
+                          ? dbits(dabs(dT)) + (28ull << 52) <= dbits(dabs(t)) || !finite_bits(dT)
+                          : !(dabs(dT) > tol * dabs(t));
+    if (done) break;
   }
   if (it == maxit) st |= ST_NEWTON_FAIL;
   T = t;
   const double Cv = fma(t, fma(t, fma(t, fma(t, c4, c3), c2), c1), K1);
   const double Cp = Cv + W;
   p = RU * W * t;
-  c = sqrt(Cp * p * rrho * rcp(Cv));
-  if (!(rho > 0.0) || !(t > 0.0) || !(p > 0.0)) st |= ST_NONPOSITIVE;
+  c = speed(Cp, p, rrho, Cv);
+  if (!positive_bits(rho) || !positive_bits(t) || !positive_bits(p)) st |= ST_NONPOSITIVE;
   if (!finite_bits(t) || !finite_bits(p) || !finite_bits(c) || !finite_bits(u[3])) st |= ST_NONFINITE;
   return st;
 }

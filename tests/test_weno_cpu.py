@@ -121,3 +121,55 @@ def test_reciprocal_and_conversion(lib):
         assert zi == 64 - xi.bit_length()
         assert abs(Q(yi) - Q(2 ** 127, xi << zi)) <= 8
         assert 0 <= Q(xi, 2 ** 64) - Q(bi) < Q(xi, 2 ** 64) * Q(2) ** -52
+
+
+def _functions(lib, x):
+    x = np.ascontiguousarray(x, dtype=np.float64)
+    out = [np.zeros(x.size) for _ in range(3)]
+    lib.wh_functions(x.size, _ptr(x), *[_ptr(o) for o in out])
+    return out
+
+
+def test_exponential_logarithm_reciprocal(lib):
+    """exp within 0.9 units in the last place (half an ulp of rounding, the
+    argument cut at 2^-54, the power of two good to 2^-57), ln within 2^-53
+    absolute plus half an ulp, 1/x within 0.51."""
+    mp = pytest.importorskip("mpmath")
+    mp.mp.prec = 160
+    rng = np.random.default_rng(5)
+    x = np.concatenate([rng.uniform(-707.9, 707.9, 3000), rng.uniform(-40, 40, 3000), rng.normal(0, 1e-3, 500),
+                        [0.0, -0.0, 1e-300, -1e-300, 5e-324, 1.0, -1.0, 512.0, -512.0, 511.99999, np.log(2.0)]])
+    e, _, _ = _functions(lib, x)
+    for xi, ei in zip(x, e):
+        assert abs(mp.mpf(float(ei)) - mp.exp(mp.mpf(float(xi)))) <= 0.9 * np.spacing(ei)
+    t = np.concatenate([rng.uniform(2, 1e4, 4000), 10.0 ** rng.uniform(0.31, 300, 1000), 2.0 ** np.arange(1, 1000, 37),
+                        np.nextafter(2.0 ** np.arange(2, 1000, 37), 0.0)])
+    _, l, _ = _functions(lib, t)
+    for ti, li in zip(t, l):
+        assert abs(mp.mpf(float(li)) - mp.log(mp.mpf(float(ti)))) <= 0.5 * np.spacing(li) + 2.0 ** -53 * max(1.0, li / 512)
+    y = 10.0 ** rng.uniform(-300, 300, 4000) * rng.choice([-1.0, 1.0], 4000) * rng.uniform(1, 2, 4000)
+    y = np.concatenate([y, 2.0 ** np.arange(-1000, 1000, 41), np.nextafter(2.0 ** np.arange(-1000, 1000, 41), 0.0)])
+    _, _, r = _functions(lib, y)
+    for yi, ri in zip(y, r):
+        assert abs(Q(float(ri)) - 1 / Q(float(yi))) <= Q(51, 100) * Q(float(np.spacing(abs(ri))))
+    _, _, r = _functions(lib, np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 1e-310, 8e307]))
+    assert np.isnan(r[:6]).all() and r[6] == 0.0
+
+
+def test_square_root_and_signed_conversion(lib):
+    rng = np.random.default_rng(6)
+    d = rng.integers(2 ** 62, 2 ** 64, 20000, dtype=np.uint64, endpoint=False)
+    d = np.concatenate([d, np.array([2 ** 62, 2 ** 62 + 1, 2 ** 63, 2 ** 64 - 1, 2 ** 63 - 1], dtype=np.uint64)])
+    s = np.zeros(d.size, np.uint64)
+    lib.wh_sqrt(d.size, _ptr(d), _ptr(s))
+    for di, si in zip(d.tolist(), s.tolist()):
+        # within 16 units: s^2 against d 2^64
+        assert (si - 16) ** 2 <= di << 64 <= (si + 16) ** 2
+    a = rng.integers(-2 ** 62, 2 ** 62, 5000) >> rng.integers(0, 62, 5000)
+    a = np.concatenate([a, [0, 1, -1, 2 ** 31, 2 ** 32, -2 ** 32, 2 ** 62, -2 ** 62, 2 ** 32 - 1]])
+    for e in (0, -1000, 900):
+        x = np.zeros(a.size)
+        lib.wh_signed(a.size, _ptr(a), e, _ptr(x))
+        for ai, xi in zip(a.tolist(), x.tolist()):
+            want = Q(ai) * Q(2) ** e
+            assert abs(Q(xi) - want) <= Q(float(np.spacing(abs(xi)))) / 2

@@ -32,6 +32,22 @@ void wh_faces(int n, int slide, const double* Fp, const double* Fm, double eps, 
   }
 }
 
+// e^x, ln x and 1/x, elementwise.
+void wh_functions(int n, const double* x, double* e, double* l, double* r) {
+  for (int i = 0; i < n; ++i) {
+    e[i] = soft::exp_double(x[i]);
+    l[i] = soft::log_double(x[i]);
+    r[i] = soft::rcp_double(x[i]);
+  }
+}
+// sqrt(d / 2^64) in units of 2^-64, and a 2^e as a double.
+void wh_sqrt(int n, const unsigned long long* d, unsigned long long* s) {
+  for (int i = 0; i < n; ++i) s[i] = soft::sqrt_q(d[i]);
+}
+void wh_signed(int n, const long long* a, int e, double* x) {
+  for (int i = 0; i < n; ++i) x[i] = soft::signed_double(a[i], e);
+}
+
 // y[i] = 2^127 / (x[i] 2^z[i]) and b[i] = x[i] 2^-64 as a double.
 void wh_soft(int n, const unsigned long long* x, unsigned long long* y, int* z, double* b) {
   for (int i = 0; i < n; ++i) {
