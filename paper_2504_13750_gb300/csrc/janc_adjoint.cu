@@ -42,7 +42,7 @@ namespace janc {
 // RHS vector-Jacobian product.
 // ---------------------------------------------------------------------------
 // Face pass, tiled like the forward face-flux kernel. A block takes
-// VLINES grid lines by VFACES (16, or 8 on small grids) consecutive faces
+// vlines_of grid lines by VFACES (16, or 8 on small grids) consecutive faces
 // along them (x tiles first, then y tiles) and stages the cotangent mu of L
 // for them; every thread owns one (variable, line) and walks its faces. At
 // face t, L_i = -(F_{i+1/2} - F_{i-1/2}) / h gives the face value the
@@ -65,7 +65,8 @@ namespace janc {
 // Two forms: k_adj_faces recomputes the reconstructions from the staged
 // cells; k_adj_faces_lin reads the derivatives the forward stored
 // (launch_face_flux_lin) and only forms the sums.
-constexpr int VLINES = 8;
+// Lines of a tile: 8, but 16 for 6 variables, whose 8 would fill one and a half warps.
+__host__ __device__ constexpr int vlines_of(int nv) { return nv == 6 ? 16 : 8; }
 
 // The per-position sums of one (variable, line) as its faces pass.
 struct EdgeSums {
@@ -105,13 +106,13 @@ struct EdgeSums {
 struct VjpTile {
   bool xdir;
   int f0, l0, nlines, nfaces, ncell, bc_lo, bc_hi, nmom;
-  __device__ __forceinline__ VjpTile(const GridDev& g, int blk, int nbx, int ntx_x, int ntx_y, int vfaces) {
+  __device__ __forceinline__ VjpTile(const GridDev& g, int blk, int nbx, int ntx_x, int ntx_y, int vlines, int vfaces) {
     xdir = blk < nbx;
     const int tile = xdir ? blk : blk - nbx;
     const int ntl = xdir ? ntx_x : ntx_y;
     const int ta = tile % ntl, tb = tile / ntl;
     f0 = xdir ? ta * vfaces : tb * vfaces;
-    l0 = xdir ? tb * VLINES : ta * VLINES;
+    l0 = xdir ? tb * vlines : ta * vlines;
     nlines = xdir ? g.ny : g.nx;
     nfaces = (xdir ? g.nx : g.ny) + 1;
     ncell = xdir ? g.nx : g.ny;
@@ -122,7 +123,7 @@ struct VjpTile {
 };
 
 // Stages mu of cells f0-1 .. f0+VFACES-1 of the tile's lines (zero outside).
-template <int NV, int VFACES>
+template <int NV, int VLINES, int VFACES>
 __device__ __forceinline__ void stage_mu(const VjpTile& T, const double* __restrict__ mu, const GridDev& g,
                                          double (*sMu)[VLINES][VFACES + 1]) {
   const long long n = g.n;
@@ -150,15 +151,15 @@ __device__ __forceinline__ double* gf_base(const VjpTile& T, double* GFx, double
 }
 
 template <int NV, int VFACES>
-__global__ void __launch_bounds__(VLINES * NV) k_adj_faces(StateView S, const double* __restrict__ alpha2,
+__global__ void __launch_bounds__(vlines_of(NV) * NV) k_adj_faces(StateView S, const double* __restrict__ alpha2,
                                                            const double* __restrict__ mu, double mu_scale,
                                                            double* __restrict__ GFx, double* __restrict__ GFy,
                                                            GridDev g, int nbx, int ntx_x, int ntx_y) {
-  constexpr int VWIN = VFACES + 5;
+  constexpr int VWIN = VFACES + 5, VLINES = vlines_of(NV);
   __shared__ double sU[NV][VLINES][VWIN];
   __shared__ double sLp[VLINES][VWIN], sLm[VLINES][VWIN], sHp[VLINES][VWIN], sHpu[VLINES][VWIN];
   __shared__ double sMu[NV][VLINES][VFACES + 1];
-  const VjpTile T(g, blockIdx.x, nbx, ntx_x, ntx_y, VFACES);
+  const VjpTile T(g, blockIdx.x, nbx, ntx_x, ntx_y, VLINES, VFACES);
   const long long n = g.n;
   const int nx = g.nx;
   const double ha = 0.5 * alpha2[T.xdir ? 0 : 1];
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(VLINES * NV) k_adj_faces(StateView S, const do
       sU[k][line][w] = v;
     }
   }
-  stage_mu<NV, VFACES>(T, mu, g, sMu);
+  stage_mu<NV, VLINES, VFACES>(T, mu, g, sMu);
   __syncthreads();
 
   const int var = threadIdx.x / VLINES;
@@ -215,9 +216,9 @@ __global__ void __launch_bounds__(VLINES * NV) k_adj_faces(StateView S, const do
     const double phi = rh * (ml[t + 1] - ml[t]);
     double d[8];
     const weno::Weights wp = P.weights_plus();
-    weno::derivative_plus(P, wp, weno::Coef(wp), d);
+    weno::derivative_plus(P, wp, P.mean_plus(wp), d);
     const weno::Weights wm = M.weights_minus();
-    weno::derivative_minus(M, wm, weno::Coef(wm), d + 4);
+    weno::derivative_minus(M, wm, M.mean_minus(wm), d + 4);
     E.add(phi, d);
     E.finish_face(phi, gbase + (long long)t * pstride, pstride);
     if (t + 1 < nf) {
@@ -229,13 +230,14 @@ __global__ void __launch_bounds__(VLINES * NV) k_adj_faces(StateView S, const do
 }
 
 template <int NV, int VFACES>
-__global__ void __launch_bounds__(VLINES * NV) k_adj_faces_lin(const double* __restrict__ lin,
+__global__ void __launch_bounds__(vlines_of(NV) * NV) k_adj_faces_lin(const double* __restrict__ lin,
                                                                const double* __restrict__ mu, double mu_scale,
                                                                double* __restrict__ GFx, double* __restrict__ GFy,
                                                                GridDev g, int nbx, int ntx_x, int ntx_y) {
+  constexpr int VLINES = vlines_of(NV);
   __shared__ double sMu[NV][VLINES][VFACES + 1];
-  const VjpTile T(g, blockIdx.x, nbx, ntx_x, ntx_y, VFACES);
-  stage_mu<NV, VFACES>(T, mu, g, sMu);
+  const VjpTile T(g, blockIdx.x, nbx, ntx_x, ntx_y, VLINES, VFACES);
+  stage_mu<NV, VLINES, VFACES>(T, mu, g, sMu);
   __syncthreads();
   const int var = threadIdx.x / VLINES;
   const int line = threadIdx.x % VLINES;
@@ -1323,7 +1325,7 @@ template <int NS>
 static cudaError_t rhs_vjp_t(const StateView& S, const double* alpha2_dev, const VjpIO& io, double* CFx, double* CFy,
                              double* scratch, const GridDev& g, const MechDev* mech, const double* lin, bool fresh,
                              bool src, const double* src_keep, cudaStream_t st) {
-  constexpr int NV = NS + 3;
+  constexpr int NV = NS + 3, VLINES = vlines_of(NV);
   const int nb = adj_cell_blocks(g);
   double* adj_alpha = scratch;
   unsigned long long* part_mx = (unsigned long long*)((char*)scratch + 256);

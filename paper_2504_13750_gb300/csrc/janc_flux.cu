@@ -4,7 +4,7 @@
 // layers of the text after Eq. 4.11 produced on the fly during the tile load.
 //
 // One launch covers both directions: blocks [0, nbx) take x-face tiles and the
-// rest take y-face tiles. A tile is LINES grid lines (rows for x, columns for
+// rest take y-face tiles. A tile is lines_of(NV) grid lines (rows for x, columns for
 // y) by 32 consecutive faces along them (16 or 8 on grids too small to fill
 // the GPU with 32-face tiles; the batched launch always uses 32). Its cells,
 // with the 5-cell stencil
@@ -14,11 +14,13 @@
 // per point instead of once per face, and each thread carries two independent
 // dependency chains.
 //
-// Bound: the FP64 pipe starts one warp instruction every 16 clocks, so the
-// nonlinear weights are formed on the integer pipes (janc_weno.cuh) and a face
-// of one variable takes 14 FP64 instructions for both signs (67 when the
-// weights were FP64 too). 2048 x 256 with 12 variables, both directions:
-// 1.73 ms a launch before, 0.60 ms now.
+// Bound: instruction issue. The FP64 pipe starts one warp instruction every 16
+// clocks, so the nonlinear weights and the weighted sums are formed on the
+// integer pipes (janc_weno.cuh): a face of one variable takes about 800
+// instructions, 8 of them FP64 (67 FP64 when all of it was). 2048 x 256 with 12
+// variables, both directions and their divergence: 1.73 ms then, 0.54 ms now.
+// The loop is not unrolled: by 2 it took 0.59 ms, by 3 0.67 ms (instruction
+// fetch).
 #include <atomic>
 
 #include "janc_device.cuh"
@@ -27,7 +29,14 @@
 
 namespace janc {
 
-constexpr int LINES = 8;
+// Lines of a tile. A block has lines x variables threads: 96 for 12 variables;
+// 6 variables take 16 lines, as 8 would fill one and a half warps
+// (1000 x 400: 4.68 ms for four steps with 8 lines, 4.07 with 16 and the sums
+// on integers).
+__host__ __device__ constexpr int lines_of(int nv) { return nv == 6 ? 16 : 8; }
+// Blocks an SM is asked to hold: 15 or 16 warps, so 128 registers a thread;
+// 132 would leave room for 12 warps (0.589 ms where 15 take 0.557).
+__host__ __device__ constexpr int blocks_of(int nv) { return 512 / (lines_of(nv) * nv); }
 constexpr int FACES = 32;  // faces per tile of the batched launch and of large grids
 
 // One tile of the face-flux launch (FC faces per line); `blk` is the tile's
@@ -42,7 +51,7 @@ __device__ __forceinline__ void face_flux_tile(const StateView& S, const unsigne
                                                double* __restrict__ Fx, double* __restrict__ Gy, const GridDev& g,
                                                int blk, int nbx, int ntx_x, int ntx_y, double* smem,
                                                double* __restrict__ lin = nullptr) {
-  constexpr int WIN = FC + 5;
+  constexpr int WIN = FC + 5, LINES = lines_of(NV);
   double* sU = smem;                       // [NV][LINES][WIN]
   double* sLp = sU + NV * LINES * WIN;     // lambda+ = (u_n + alpha) / 2
   double* sLm = sLp + LINES * WIN;         // lambda- = (u_n - alpha) / 2
@@ -135,7 +144,7 @@ __device__ __forceinline__ void face_flux_tile(const StateView& S, const unsigne
 }
 
 template <int NV, int FC, bool HALO>
-__global__ void __launch_bounds__(LINES * NV) k_face_flux(StateView S, const unsigned long long* __restrict__ alpha,
+__global__ void __launch_bounds__(lines_of(NV) * NV, blocks_of(NV)) k_face_flux(StateView S, const unsigned long long* __restrict__ alpha,
                                                           double* __restrict__ Fx, double* __restrict__ Gy,
                                                           GridDev g, int nbx, int ntx_x, int ntx_y) {
   extern __shared__ double smem[];
@@ -146,7 +155,7 @@ __global__ void __launch_bounds__(LINES * NV) k_face_flux(StateView S, const uns
 // reconstruction with respect to its window differences in `lin` (the
 // discrete adjoint's face-derivative store).
 template <int NV, int FC>
-__global__ void __launch_bounds__(LINES * NV) k_face_flux_lin(StateView S, const unsigned long long* __restrict__ alpha,
+__global__ void __launch_bounds__(lines_of(NV) * NV) k_face_flux_lin(StateView S, const unsigned long long* __restrict__ alpha,
                                                               double* __restrict__ Fx, double* __restrict__ Gy,
                                                               double* __restrict__ lin, GridDev g, int nbx, int ntx_x,
                                                               int ntx_y) {
@@ -157,7 +166,7 @@ __global__ void __launch_bounds__(LINES * NV) k_face_flux_lin(StateView S, const
 // Batched form: a persistent grid walks the flattened (request, tile) list;
 // request r owns entries [first[r], first[r+1]).
 template <int NV>
-__global__ void __launch_bounds__(LINES * NV) k_face_flux_batch(const BatchReq* __restrict__ reqs,
+__global__ void __launch_bounds__(lines_of(NV) * NV, blocks_of(NV)) k_face_flux_batch(const BatchReq* __restrict__ reqs,
                                                                 const int* __restrict__ first, int nreq, int state) {
   extern __shared__ double smem[];
   const int total = first[nreq];
@@ -172,7 +181,7 @@ __global__ void __launch_bounds__(LINES * NV) k_face_flux_batch(const BatchReq* 
 
 template <int NV, int FC = FACES>
 static size_t flux_smem_bytes() {
-  return sizeof(double) * (size_t)(NV + 4) * LINES * (FC + 5);
+  return sizeof(double) * (size_t)(NV + 4) * lines_of(NV) * (FC + 5);
 }
 
 int sm_count() {
@@ -204,10 +213,11 @@ cudaError_t set_attr_once(const void* func, cudaFuncAttribute attr, int value, s
 }
 
 // Tiles of FC faces: x tiles first, then y tiles.
-static void tiles_of(const GridDev& g, int fc, int* nbx, int* ntx_x, int* ntx_y, int* total) {
+static void tiles_of(const GridDev& g, int nv, int fc, int* nbx, int* ntx_x, int* ntx_y, int* total) {
+  const int lines = lines_of(nv);
   *ntx_x = (g.nx + 1 + fc - 1) / fc;
-  const int nty_x = (g.ny + LINES - 1) / LINES;
-  *ntx_y = (g.nx + LINES - 1) / LINES;
+  const int nty_x = (g.ny + lines - 1) / lines;
+  *ntx_y = (g.nx + lines - 1) / lines;
   const int nty_y = (g.ny + 1 + fc - 1) / fc;
   *nbx = *ntx_x * nty_x;
   *total = *nbx + *ntx_y * nty_y;
@@ -217,13 +227,13 @@ template <int NV, int FC, bool HALO>
 static cudaError_t launch_face_flux_fc(const StateView& S, const unsigned long long* alpha, double* Fx, double* Gy,
                                        const GridDev& g, cudaStream_t st) {
   int nbx, ntx_x, ntx_y, total;
-  tiles_of(g, FC, &nbx, &ntx_x, &ntx_y, &total);
+  tiles_of(g, NV, FC, &nbx, &ntx_x, &ntx_y, &total);
   const size_t smem = flux_smem_bytes<NV, FC>();
   static std::atomic<unsigned long long> attr_done{0};
   cudaError_t e = set_attr_once((const void*)k_face_flux<NV, FC, HALO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem, &attr_done);
   if (e != cudaSuccess) return e;
-  k_face_flux<NV, FC, HALO><<<total, LINES * NV, smem, st>>>(S, alpha, Fx, Gy, g, nbx, ntx_x, ntx_y);
+  k_face_flux<NV, FC, HALO><<<total, lines_of(NV) * NV, smem, st>>>(S, alpha, Fx, Gy, g, nbx, ntx_x, ntx_y);
   return cudaGetLastError();
 }
 
@@ -232,19 +242,19 @@ static cudaError_t launch_face_flux_fc(const StateView& S, const unsigned long l
 // and a larger share of stencil margin; on small grids, whose launches are a
 // fraction of a wave and latency-bound, the blocks win (measured on one
 // GB300: 256 x 32 runs best at 8, 512 x 64 at 16, 4096 x 512 at 32).
-static int flux_tile_faces(const GridDev& g) {
+static int flux_tile_faces(const GridDev& g, int nv) {
   const int sms = sm_count();
   int nbx, ntx_x, ntx_y, total;
-  tiles_of(g, 32, &nbx, &ntx_x, &ntx_y, &total);
+  tiles_of(g, nv, 32, &nbx, &ntx_x, &ntx_y, &total);
   if (total >= 8 * sms) return 32;
-  tiles_of(g, 16, &nbx, &ntx_x, &ntx_y, &total);
+  tiles_of(g, nv, 16, &nbx, &ntx_x, &ntx_y, &total);
   return total >= 2 * sms ? 16 : 8;
 }
 
 template <int NV, bool HALO>
 static cudaError_t launch_face_flux_h(const StateView& S, const unsigned long long* alpha, double* Fx, double* Gy,
                                       const GridDev& g, cudaStream_t st) {
-  switch (flux_tile_faces(g)) {
+  switch (flux_tile_faces(g, NV)) {
     case 32: return launch_face_flux_fc<NV, 32, HALO>(S, alpha, Fx, Gy, g, st);
     case 16: return launch_face_flux_fc<NV, 16, HALO>(S, alpha, Fx, Gy, g, st);
     default: return launch_face_flux_fc<NV, 8, HALO>(S, alpha, Fx, Gy, g, st);
@@ -262,20 +272,20 @@ template <int NV, int FC>
 static cudaError_t launch_face_flux_lin_fc(const StateView& S, const unsigned long long* alpha, double* Fx, double* Gy,
                                            double* lin, const GridDev& g, cudaStream_t st) {
   int nbx, ntx_x, ntx_y, total;
-  tiles_of(g, FC, &nbx, &ntx_x, &ntx_y, &total);
+  tiles_of(g, NV, FC, &nbx, &ntx_x, &ntx_y, &total);
   const size_t smem = flux_smem_bytes<NV, FC>();
   static std::atomic<unsigned long long> attr_done{0};
   cudaError_t e = set_attr_once((const void*)k_face_flux_lin<NV, FC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem, &attr_done);
   if (e != cudaSuccess) return e;
-  k_face_flux_lin<NV, FC><<<total, LINES * NV, smem, st>>>(S, alpha, Fx, Gy, lin, g, nbx, ntx_x, ntx_y);
+  k_face_flux_lin<NV, FC><<<total, lines_of(NV) * NV, smem, st>>>(S, alpha, Fx, Gy, lin, g, nbx, ntx_x, ntx_y);
   return cudaGetLastError();
 }
 
 template <int NV>
 static cudaError_t launch_face_flux_lin_t(const StateView& S, const unsigned long long* alpha, double* Fx, double* Gy,
                                           double* lin, const GridDev& g, cudaStream_t st) {
-  switch (flux_tile_faces(g)) {
+  switch (flux_tile_faces(g, NV)) {
     case 32: return launch_face_flux_lin_fc<NV, 32>(S, alpha, Fx, Gy, lin, g, st);
     case 16: return launch_face_flux_lin_fc<NV, 16>(S, alpha, Fx, Gy, lin, g, st);
     default: return launch_face_flux_lin_fc<NV, 8>(S, alpha, Fx, Gy, lin, g, st);
@@ -297,8 +307,8 @@ cudaError_t launch_face_flux_lin(int nv, const StateView& S, const unsigned long
   }
 }
 
-void face_flux_tiles(const GridDev& g, int* nbx, int* ntx_x, int* ntx_y, int* total) {
-  tiles_of(g, FACES, nbx, ntx_x, ntx_y, total);
+void face_flux_tiles(const GridDev& g, int nv, int* nbx, int* ntx_x, int* ntx_y, int* total) {
+  tiles_of(g, nv, FACES, nbx, ntx_x, ntx_y, total);
 }
 
 template <int NV>
@@ -311,7 +321,7 @@ static cudaError_t launch_face_flux_batch_t(const BatchReq* reqs, const int* fir
   if (e != cudaSuccess) return e;
   const int sms = sm_count();
   const int grid = total < sms * 8 ? total : sms * 8;
-  if (grid > 0) k_face_flux_batch<NV><<<grid, LINES * NV, smem, st>>>(reqs, first, nreq, state);
+  if (grid > 0) k_face_flux_batch<NV><<<grid, lines_of(NV) * NV, smem, st>>>(reqs, first, nreq, state);
   return cudaGetLastError();
 }
 

@@ -71,7 +71,7 @@ cudaError_t launch_set_conserved(int ns, const StateView& S, const double* T0, c
                                  unsigned long long* alpha_out, int* status, cudaStream_t st);
 // Batched launches over a flattened (request, block) list; first[0..nreq]
 // holds each request's first entry, first[nreq] the total (device memory).
-void face_flux_tiles(const GridDev& g, int* nbx, int* ntx_x, int* ntx_y, int* total);
+void face_flux_tiles(const GridDev& g, int nv, int* nbx, int* ntx_x, int* ntx_y, int* total);
 void update_blocks(const GridDev& g, int* ubx, int* uby);
 int chem_blocks(const GridDev& g);
 cudaError_t launch_batch_prep(BatchReq* reqs, int nreq, cudaStream_t st);

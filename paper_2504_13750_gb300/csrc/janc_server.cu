@@ -150,7 +150,7 @@ void fill_batchreq(janc_server_s* s, Req* r) {
   b.ctl.source = 0;
   b.ctl.hmin = g.dx < g.dy ? g.dx : g.dy;
   int tot_f;
-  face_flux_tiles(g, &b.nbx, &b.ntx_x, &b.ntx_y, &tot_f);
+  face_flux_tiles(g, s->nv, &b.nbx, &b.ntx_x, &b.ntx_y, &tot_f);
   update_blocks(g, &b.ubx, &b.uby);
 }
 
@@ -220,7 +220,7 @@ int upload(janc_server_s* s) {
     r->br.fresh = r->fresh;
     hb[q] = r->br;
     int nbx, ntx, nty, tf;
-    face_flux_tiles(r->br.g, &nbx, &ntx, &nty, &tf);
+    face_flux_tiles(r->br.g, s->nv, &nbx, &ntx, &nty, &tf);
     hf[q] = acc[0];
     hf[(s->max_active + 1) + q] = acc[1];
     hf[2 * (s->max_active + 1) + q] = acc[2];

@@ -77,6 +77,17 @@ JANC_HD u64 shl(u64 x, int n) {
 #endif
 }
 
+// x / 2^n for n >= 0, rounded down.
+JANC_HD long long sar(long long x, int n) {
+#ifdef __CUDA_ARCH__
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+  return r;
+#else
+  return x >> (n > 63 ? 63 : n);
+#endif
+}
+
 // a b / 2^64, at most 2 below the exact quotient (the product of the low
 // words is left out). 3 wide products.
 JANC_HD u64 mulhi(u64 a, u64 b) {
@@ -320,6 +331,20 @@ JANC_HD double signed_double(long long a, int e) {
   const int z = leading_zeros(h);
   const u64 b = bits_of(round_double(shl(((u64)h << 32) | l, z), e - z + 63));
   return a == 0 ? 0.0 : double_of(((u64)(hi32(b) | (a < 0 ? 0x80000000u : 0u)) << 32) | lo32(b));
+}
+
+// a 2^e rounded to nearest, 0 below the normal range. No check against overflow.
+JANC_HD double scaled_double(long long a, int e) {
+  u64 m = a < 0 ? 0ull - (u64)a : (u64)a;
+  if (hi32(m) == 0) {
+    m <<= 32;
+    e -= 32;
+  }
+  const int z = leading_zeros(hi32(m));  // 158 for 0
+  const int x = 1085 + e - z;
+  m = shl(m, z);
+  const u64 b = (m >> 11) + ((m >> 10) & 1) + ((u64)((u32)x << 20 | ((u32)hi32((u64)a) & 0x80000000u)) << 32);
+  return double_of(x < 0 || m == 0 ? 0ull : b);
 }
 
 // sqrt(d / 2^64) for d in [2^62, 2^64), in units of 2^-64, within 2^-60: a float

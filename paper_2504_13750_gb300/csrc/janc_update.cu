@@ -346,7 +346,7 @@ __global__ void k_rhs_L(int nv, const double* __restrict__ Fx, const double* __r
   const int j = (int)(idx / g.nx), i = (int)(idx % g.nx);
   const double dF = Fx[((long long)k * g.ny + j) * (g.nx + 1) + i + 1] - Fx[((long long)k * g.ny + j) * (g.nx + 1) + i];
   const double dG = Gy[((long long)k * (g.ny + 1) + j + 1) * g.nx + i] - Gy[((long long)k * (g.ny + 1) + j) * g.nx + i];
-  L[q] = -fma(dF, g.rdx, dG * g.rdy);
+  L[q] = fma(-dF, g.rdx, -(dG * g.rdy));
 }
 
 cudaError_t launch_rhs_L(int nv, const double* Fx, const double* Gy, double* L, const GridDev& g, cudaStream_t st) {

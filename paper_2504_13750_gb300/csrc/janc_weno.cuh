@@ -2,14 +2,18 @@
 // single-grid, the block (AMR) and the adjoint face kernels.
 //
 // The reconstruction costs the FP64 pipe little: with D_j = F_j - F_{j-1} the
-// differences of the five values of a window, the face value is
-//   F_2 + c1 D1 + c2 D2 + c3 D3 + c4 D4,
-//   c1 = -w0/3, c2 = (w1 + 5 w0)/6, c3 = (w1 + 2 w2)/3, c4 = -w2/6
-// with the nonlinear weights w_k of the three substencils. Only D_j, the
-// products with c_m and their sum are FP64 operations (14 per face for both
-// split signs). The weights are formed on 64-bit integers (janc_soft.cuh),
-// accurate to about 2^-55, which the FP64 pipe's own evaluation (about 2^-51)
-// does not reach.
+// differences of the five values of a window, the face value is F_2 plus
+//   r = (w0 Q0 + w1 Q1 + w2 Q2) / 6,
+//   Q0 = 5 D2 - 2 D1, Q1 = D2 + 2 D3, Q2 = 4 D3 - D4
+// with the nonlinear weights w_k of the three substencils. Only the split
+// fluxes, D_j, and the final products and sums are FP64 operations (8 per face
+// for both split signs). The weights and the weighted sum of the Q_k are formed
+// on 64-bit integers (janc_soft.cuh): weights accurate to about 2^-55, the sum
+// to 2^-51 or better of its largest term, which the FP64 pipe's own evaluation
+// (about 2^-51) does not reach. 2048 x 256, 12 variables, both directions:
+// 0.597 ms with the coefficients of the D_j as doubles (14 FP64 instructions a
+// face), 0.557 ms with the sum on integers; with the derivatives (1000 x 400,
+// 6 variables) 1.05 and 0.56 ms.
 //
 // The smoothness indicators are quadratic forms of adjacent differences,
 //   3 beta_0 = 4 D1^2 - 11 D1 D2 + 10 D2^2,
@@ -65,16 +69,29 @@ struct Eps {
   }
 };
 
-// One difference: its mantissa in [2^63, 2^64), exponent field and square.
+// One difference: its mantissa in [2^63, 2^64), exponent field, sign (all ones
+// if negative) and square.
 struct Diff {
   u64 m, sq;
-  int e;
+  int e, neg;
   JANC_HD void set(double D) {
     const u64 b = bits_of(D);
     e = (int)(hi32(b) >> 20) & 0x7ff;
+    neg = (int)hi32(b) >> 31;
     m = (b << 11) | (1ull << 63);
     sq = sqhi(m);
   }
+};
+JANC_HD long long with_sign(u64 x, int neg) {
+  const u64 s = ((u64)(u32)neg << 32) | (u32)neg;
+  return (long long)((x ^ s) - s);
+}
+
+// An adjacent pair of differences as signed integers below 2^58 in units of
+// 2^(e - 1080), e the larger exponent field.
+struct Pair {
+  long long a, b;
+  int e;
 };
 
 // 3 (beta + epsilon) of the pair (a, b) as substencil 0, 1 and 2, in units of
@@ -82,27 +99,28 @@ struct Diff {
 struct Forms {
   Num c0, c1, c2;
 };
-JANC_HD Forms pair_forms(double Da, double Db, const Diff& a, const Diff& b, const Eps& eps) {
-  int e = a.e > b.e ? a.e : b.e;
-  e = e > eps.e_min ? e : eps.e_min;
+JANC_HD Forms pair_forms(const Diff& a, const Diff& b, const Eps& eps, Pair& p) {
+  p.e = a.e > b.e ? a.e : b.e;
+  p.a = with_sign(shr(a.m, p.e - a.e + 6), a.neg);
+  p.b = with_sign(shr(b.m, p.e - b.e + 6), b.neg);
+  const int e = p.e > eps.e_min ? p.e : eps.e_min;
   const int da = e - a.e, db = e - b.e;
   const u64 A = shr(a.sq, 2 * da + 5), B = shr(b.sq, 2 * db + 5);
   const u64 C = shr(mulhi(a.m, b.m), da + db + 5);
-  const bool opposite = (int)(hi32(bits_of(Da)) ^ hi32(bits_of(Db))) < 0;
-  const u64 X = opposite ? C : 0ull - C;  // -D_a D_b
+  const u64 X = (u64)with_sign(C, ~(a.neg ^ b.neg));  // -D_a D_b
   const u64 t = ((A + B) << 2) + shr(eps.n, 2 * (e - eps.e_min));
   const u64 u = t + 11 * X;
   return Forms{normal(u + 6 * B, 2 * e), normal(t + 5 * X, 2 * e), normal(u + 6 * A, 2 * e)};
 }
 
 // Weights of substencils with indicators s0, s1, s2 and linear weights
-// 1 : 6 : 3, a sixth of each: w0 = u0 2^(x - 5 - 2 d0), w1 = 3 u1 2^(x - 4 - 2 d1),
-// w2 = 3 u2 2^(x - 5 - 2 d2), all times 2^-64, with u_k in [2^59, 2^64): each
-// weight keeps its relative accuracy however small it is. The weights are
-// 1/s_k^2 up to a common factor; with s0^2 s1^2 s2^2 as that factor they are
-// the squares of the products p12 = s1 s2 and so on (upper halves).
+// 1 : 6 : 3. The weights are 1/s_k^2 up to a common factor; with s0^2 s1^2 s2^2
+// as that factor they are the squares u_k 2^(-2 d_k) of the products
+// p12 = s1 s2 and so on (upper halves), each with its own exponent, so that a
+// weight keeps its relative accuracy however small it is. y 2^x is 2^127 over
+// 1.5 times their sum / 16.
 struct Weights {
-  u64 u0, u1, u2, p12, p02, p01;
+  u64 u0, u1, u2, p12, p02, p01, y;
   int x, d0, d1, d2;
   JANC_HD Weights(const Num& s0, const Num& s1, const Num& s2) {
     p12 = mulhi(s1.n, s2.n);
@@ -117,52 +135,76 @@ struct Weights {
     u1 = sqhi(p02);
     u2 = sqhi(p01);
     const u64 s = shr(u0, 2 * d0 + 4) + 3 * (shr(u1, 2 * d1 + 3) + shr(u2, 2 * d2 + 4));
-    const u64 y = recip(s + (s >> 1), &x);  // 2^127 / (1.5 s 2^x)
-    u0 = mulhi(u0, y);
-    u1 = mulhi(u1, y);
-    u2 = mulhi(u2, y);
+    y = recip(s + (s >> 1), &x);
   }
 };
 
-// The sizes |c1|, c2, c3, |c4| of the coefficients in the stencil's own
-// direction. c2 and c3 are sums of two weights aligned to the larger one.
+// u q / 2^64 for signed q, at most 3 below the exact quotient.
+JANC_HD long long mulhi_signed(u64 u, long long q) {
+  return (long long)(mulhi(u, (u64)q) - (q < 0 ? u : 0ull));
+}
+
+// The weighted mean r = n y of the substencils' offsets (Q_k / 6): Q_k as
+// integers in units of 2^(e_k - 1080) below 7 2^58, 3 2^58, 5 2^58. Their
+// products with the weights are aligned to the largest and summed below 2^63.
+// Not finite where a difference was not.
+struct Mean {
+  double n, y;
+  JANC_HD Mean(const Weights& w, long long q0, int e0, long long q1, int e1, long long q2, int e2) {
+    const int t0 = e0 - 2 * w.d0, t1 = e1 - 2 * w.d1 + 2, t2 = e2 - 2 * w.d2 + 1;  // weights 1, 4 (1.5), 2 (1.5)
+    int t = t0 > t1 ? t0 : t1;
+    t = t > t2 ? t : t2;
+    const long long v = sar(mulhi_signed(w.u1, q1), t - t1) + sar(mulhi_signed(w.u2, q2), t - t2);
+    n = scaled_double(sar(mulhi_signed(w.u0, q0), t - t0) + v + (v >> 1), t + w.x - 1085);
+    int e = e0 > e1 ? e0 : e1;
+    e = e > e2 ? e : e2;
+    if (e > 2000) n = double_of(0x7ff8000000000000ull);
+    y = round_double(w.y, -1);
+  }
+};
+
+// The sizes |c1|, c2, c3, |c4| of the derivatives of r at fixed weights
+// (r = -c1 D1 + c2 D2 + c3 D3 - c4 D4), in the stencil's own direction, and a
+// sixth of each weight: w0 = u0 2^(x - 5 - 2 d0), w1 = 3 u1 2^(x - 4 - 2 d1),
+// w2 = 3 u2 2^(x - 5 - 2 d2), all times 2^-64. c2 and c3 are sums of two
+// weights aligned to the larger one.
 struct Coef {
+  u64 u0, u1, u2;
   double k1, k2, k3, k4;
-  JANC_HD explicit Coef(const Weights& w) {
-    const u64 v1 = w.u1 >> 3, v2 = w.u2 >> 3;
+  JANC_HD explicit Coef(const Weights& w) : u0(mulhi(w.u0, w.y)), u1(mulhi(w.u1, w.y)), u2(mulhi(w.u2, w.y)) {
+    const u64 v1 = u1 >> 3, v2 = u2 >> 3;
     const int m = w.d0 < w.d1 ? w.d0 : w.d1, n = w.d1 < w.d2 ? w.d1 : w.d2;
-    k1 = to_double(w.u0, w.x - 4 - 2 * w.d0);
-    k2 = to_double(3 * shr(v1, 2 * (w.d1 - m)) + 5 * shr(w.u0, 2 * (w.d0 - m) + 4), w.x - 1 - 2 * m);
+    k1 = to_double(u0, w.x - 4 - 2 * w.d0);
+    k2 = to_double(3 * shr(v1, 2 * (w.d1 - m)) + 5 * shr(u0, 2 * (w.d0 - m) + 4), w.x - 1 - 2 * m);
     k3 = to_double(3 * (shr(v1, 2 * (w.d1 - n)) + shr(v2, 2 * (w.d2 - n))), w.x - 2 * n);
-    k4 = to_double(3 * (w.u2 >> 2), w.x - 3 - 2 * w.d2);
+    k4 = to_double(3 * (u2 >> 2), w.x - 3 - 2 * w.d2);
   }
 };
 
-// Sliding window of one split sign along a line: values F_2..F_4, differences
-// D1..D4 and the forms of the pairs (1 2), (2 3), (3 4) that the current and
-// the next two windows use.
+// Sliding window of one split sign along a line: values F_2..F_4, the last
+// difference, the pairs (1 2) A, (2 3) B, (3 4) C of differences and the forms
+// that the current and the next two windows use of them.
 struct Win {
-  double F2, F3, F4, D1, D2, D3, D4;
+  double F2, F3, F4;
   Diff d4;
-  Num a0, b0, c0, b1, c1, c2;  // pair (1 2) a, (2 3) b, (3 4) c
+  Pair A, B, C;
+  Num a0, b0, c0, b1, c1, c2;  // pair A: a, B: b, C: c
   JANC_HD void init(double F0, double F1, double f2, double f3, double f4, const Eps& eps) {
     F2 = f2; F3 = f3; F4 = f4;
-    D1 = sub_rn(F1, F0); D2 = sub_rn(F2, F1); D3 = sub_rn(F3, F2); D4 = sub_rn(F4, F3);
     Diff d1, d2, d3;
-    d1.set(D1); d2.set(D2); d3.set(D3); d4.set(D4);
-    a0 = pair_forms(D1, D2, d1, d2, eps).c0;
-    const Forms b = pair_forms(D2, D3, d2, d3, eps);
+    d1.set(sub_rn(F1, F0)); d2.set(sub_rn(F2, F1)); d3.set(sub_rn(F3, F2)); d4.set(sub_rn(F4, F3));
+    a0 = pair_forms(d1, d2, eps, A).c0;
+    const Forms b = pair_forms(d2, d3, eps, B);
     b0 = b.c0; b1 = b.c1;
-    const Forms c = pair_forms(D3, D4, d3, d4, eps);
+    const Forms c = pair_forms(d3, d4, eps, C);
     c0 = c.c0; c1 = c.c1; c2 = c.c2;
   }
   JANC_HD void push(double Fn, const Eps& eps) {
-    const double Dn = sub_rn(Fn, F4);
-    F2 = F3; F3 = F4; F4 = Fn;
     Diff dn;
-    dn.set(Dn);
-    const Forms f = pair_forms(D4, Dn, d4, dn, eps);
-    D1 = D2; D2 = D3; D3 = D4; D4 = Dn;
+    dn.set(sub_rn(Fn, F4));
+    F2 = F3; F3 = F4; F4 = Fn;
+    A = B; B = C;
+    const Forms f = pair_forms(d4, dn, eps, C);
     d4 = dn;
     a0 = b0; b0 = c0; c0 = f.c0;
     b1 = c1; c1 = f.c1;
@@ -170,64 +212,66 @@ struct Win {
   }
   // F+ at the right face of cell 2: substencils 0, 1, 2 from the left.
   JANC_HD Weights weights_plus() const { return Weights(a0, b1, c2); }
-  // F- at the left face of cell 2: the mirror image.
+  JANC_HD Mean mean_plus(const Weights& w) const {
+    return Mean(w, 5 * A.b - 2 * A.a, A.e, B.a + 2 * B.b, B.e, 4 * C.a - C.b, C.e);
+  }
+  // F- at the left face of cell 2: the mirror image, whose differences run
+  // backwards with the sign changed. The mean is that of the unchanged signs.
   JANC_HD Weights weights_minus() const { return Weights(c2, b1, a0); }
+  JANC_HD Mean mean_minus(const Weights& w) const {
+    return Mean(w, 5 * C.a - 2 * C.b, C.e, B.b + 2 * B.a, B.e, 4 * A.b - A.a, A.e);
+  }
 };
 
-// c1 D1 + .. + c4 D4 added to r.
-JANC_HD double offset_plus(const Win& P, const Coef& p) {
-  return fma(-p.k4, P.D4, fma(-p.k1, P.D1, fma(p.k3, P.D3, mul_rn(p.k2, P.D2))));
-}
-JANC_HD double offset_minus(const Win& M, const Coef& m, double r) {
-  return fma(m.k4, M.D1, fma(m.k1, M.D4, fma(-m.k3, M.D2, fma(-m.k2, M.D3, r))));
-}
-// F+ of window P plus F- of window M at their common face: the eight small
+// F+ of window P plus F- of window M at their common face: the two small
 // terms first, then the two centre values.
-JANC_HD double face_sum(const Win& P, const Coef& p, const Win& M, const Coef& m) {
-  return sub_rn(sub_rn(P.F2, -M.F2), -offset_minus(M, m, offset_plus(P, p)));
+JANC_HD double face_sum(const Win& P, const Mean& p, const Win& M, const Mean& m) {
+  return sub_rn(sub_rn(P.F2, -M.F2), -fma(-m.n, m.y, mul_rn(p.n, p.y)));
 }
 
 // The derivative of one reconstruction with respect to its window's
-// differences D1..D4 in the stencil's own direction (for F-: D4..D1 with the
-// sign changed): with q_k the substencils' offsets and r their weighted mean,
-// both less F_2,
-//   dr/dD_m = c_m + sum_k h_k dC_k/dD_m, h_k = -2 (w_k / C_k) (q_k - r),
-// C_k = 3 (beta_k + eps) and dC_k/dD_m linear in the pair's differences.
+// differences in the stencil's own direction, d_1..d_4: with r their weighted
+// mean of the substencils' offsets q_k = Q_k / 6,
+//   dr/dd_m = c_m + sum_k h_k dC_k/dd_m, h_k = -2 (w_k / C_k) (q_k - r),
+// C_k = 3 (beta_k + eps) and dC_k/dd_m linear in the pair's differences.
 // w_k / C_k comes from the products of the weights and one more reciprocal,
-// that of C_0 C_1 C_2.
-JANC_HD void derivative(const Num& s0, const Num& s1, const Num& s2, const Weights& w, const Coef& c, double D1,
-                        double D2, double D3, double D4, double r, double* g) {
+// that of C_0 C_1 C_2. (a_k, b_k): the pair of substencil k, first difference
+// first, in units of 2^(e_k - 1080): Q_k and dC_k/dd_m are small integer
+// combinations of them, formed on integers and converted, so that 14 FP64
+// instructions are left of 30.
+JANC_HD void derivative(const Num& s0, const Num& s1, const Num& s2, const Weights& w, const Coef& c, const Mean& r,
+                        long long a0, long long b0, int e0, long long a1, long long b1, int e1, long long a2,
+                        long long b2, int e2, double* g) {
   int z;
   const u64 y = recip(mulhi(w.p12, s0.n), &z);
   // 1 / C_0 = mulhi(p12, y) 2^(z - 127 + 2103 - e_0); twice the sixth of the weight over C_k
   const int b = w.x + z + 1 - 127 + 2103;
-  const double G0 = to_double(mulhi(w.u0, mulhi(w.p12, y)), b - 5 - 2 * w.d0 - s0.e + 64);
-  const double G1 = to_double(3 * (mulhi(w.u1, mulhi(w.p02, y)) >> 2), b - 2 - 2 * w.d1 - s1.e + 64);
-  const double G2 = to_double(3 * (mulhi(w.u2, mulhi(w.p01, y)) >> 2), b - 3 - 2 * w.d2 - s2.e + 64);
-  // 6 (r - q_k)
-  const double h0 = G0 * fma(6.0, r, fma(-5.0, D2, 2.0 * D1));
-  const double h1 = G1 * fma(6.0, r, fma(-2.0, D3, -D2));
-  const double h2 = G2 * fma(6.0, r, fma(-4.0, D3, D4));
-  double a = h0 * D1, t = h0 * D2;
-  g[0] = fma(8.0, a, fma(-11.0, t, -c.k1));
-  g[1] = fma(20.0, t, fma(-11.0, a, c.k2));
-  a = h1 * D2; t = h1 * D3;
-  g[1] = fma(8.0, a, fma(-5.0, t, g[1]));
-  g[2] = fma(8.0, t, fma(-5.0, a, c.k3));
-  a = h2 * D3; t = h2 * D4;
-  g[2] = fma(20.0, a, fma(-11.0, t, g[2]));
-  g[3] = fma(8.0, t, fma(-11.0, a, -c.k4));
+  const double G0 = to_double(mulhi(c.u0, mulhi(w.p12, y)), b - 5 - 2 * w.d0 - s0.e + 64);
+  const double G1 = to_double(3 * (mulhi(c.u1, mulhi(w.p02, y)) >> 2), b - 2 - 2 * w.d1 - s1.e + 64);
+  const double G2 = to_double(3 * (mulhi(c.u2, mulhi(w.p01, y)) >> 2), b - 3 - 2 * w.d2 - s2.e + 64);
+  const double r6 = mul_rn(mul_rn(6.0, r.n), r.y);
+  e0 -= 1080;
+  e1 -= 1080;
+  e2 -= 1080;
+  const double h0 = G0 * sub_rn(r6, scaled_double(5 * b0 - 2 * a0, e0));
+  const double h1 = G1 * sub_rn(r6, scaled_double(a1 + 2 * b1, e1));
+  const double h2 = G2 * sub_rn(r6, scaled_double(4 * a2 - b2, e2));
+  g[0] = fma(h0, scaled_double(8 * a0 - 11 * b0, e0), -c.k1);
+  g[1] = fma(h1, scaled_double(8 * a1 - 5 * b1, e1), fma(h0, scaled_double(20 * b0 - 11 * a0, e0), c.k2));
+  g[2] = fma(h2, scaled_double(20 * a2 - 11 * b2, e2), fma(h1, scaled_double(8 * b1 - 5 * a1, e1), c.k3));
+  g[3] = fma(h2, scaled_double(8 * b2 - 11 * a2, e2), -c.k4);
 }
 // The derivatives of the F+ and the F- reconstruction with respect to the
 // window's D1..D4.
-JANC_HD void derivative_plus(const Win& P, const Weights& w, const Coef& c, double* g) {
-  derivative(P.a0, P.b1, P.c2, w, c, P.D1, P.D2, P.D3, P.D4, offset_plus(P, c), g);
+JANC_HD void derivative_plus(const Win& P, const Weights& w, const Mean& r, double* g) {
+  derivative(P.a0, P.b1, P.c2, w, Coef(w), r, P.A.a, P.A.b, P.A.e, P.B.a, P.B.b, P.B.e, P.C.a, P.C.b, P.C.e, g);
 }
-JANC_HD void derivative_minus(const Win& M, const Weights& w, const Coef& c, double* g) {
-  // with the differences D'_1 = -D4 .. D'_4 = -D1; all of them negated below,
-  // which turns r - q and the products h D' but not the derivatives' values
+JANC_HD void derivative_minus(const Win& M, const Weights& w, const Mean& r, double* g) {
+  // the stencil's differences are -D4..-D1: the signs of r and q_k change, h_k
+  // times a difference does not, and neither do the derivatives' values but for
+  // the sign of dd/dD
   double t[4];
-  derivative(M.c2, M.b1, M.a0, w, c, M.D4, M.D3, M.D2, M.D1, -offset_minus(M, c, 0.0), t);
+  derivative(M.c2, M.b1, M.a0, w, Coef(w), r, M.C.b, M.C.a, M.C.e, M.B.b, M.B.a, M.B.e, M.A.b, M.A.a, M.A.e, t);
   g[0] = -t[3]; g[1] = -t[2]; g[2] = -t[1]; g[3] = -t[0];
 }
 
@@ -255,8 +299,8 @@ __device__ __forceinline__ void slide_line2(const SplitLine& L, double eps4, int
   weno::Win P, M;
   L.init(P, M, eps);
   for (int t = 0; t < nf; ++t) {
-    const weno::Coef cp(P.weights_plus()), cm(M.weights_minus());
-    out[(long long)t * stride] = weno::face_sum(P, cp, M, cm);
+    const weno::Mean rp = P.mean_plus(P.weights_plus()), rm = M.mean_minus(M.weights_minus());
+    out[(long long)t * stride] = weno::face_sum(P, rp, M, rm);
     if (t + 1 < nf) {
       P.push(L.plus(t + 5), eps);
       M.push(L.minus(t + 6), eps);
@@ -278,16 +322,16 @@ __device__ __forceinline__ void slide_line2_lin(const SplitLine& L, double eps4,
     double g[4];
     double* l = lin + (long long)t * fstride;
     const weno::Weights wp = P.weights_plus();
-    const weno::Coef cp(wp);
-    weno::derivative_plus(P, wp, cp, g);
+    const weno::Mean rp = P.mean_plus(wp);
+    weno::derivative_plus(P, wp, rp, g);
 #pragma unroll
     for (int c = 0; c < 4; ++c) l[c * cstride] = g[c];
     const weno::Weights wm = M.weights_minus();
-    const weno::Coef cm(wm);
-    weno::derivative_minus(M, wm, cm, g);
+    const weno::Mean rm = M.mean_minus(wm);
+    weno::derivative_minus(M, wm, rm, g);
 #pragma unroll
     for (int c = 0; c < 4; ++c) l[(4 + c) * cstride] = g[c];
-    out[(long long)t * stride] = weno::face_sum(P, cp, M, cm);
+    out[(long long)t * stride] = weno::face_sum(P, rp, M, rm);
     if (t + 1 < nf) {
       P.push(L.plus(t + 5), eps);
       M.push(L.minus(t + 6), eps);

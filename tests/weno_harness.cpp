@@ -25,10 +25,10 @@ void wh_faces(int n, int slide, const double* Fp, const double* Fm, double eps, 
       M.push(m[t + 6], e);
     }
     const weno::Weights wp = P.weights_plus(), wm = M.weights_minus();
-    const weno::Coef cp(wp), cm(wm);
-    sum[i] = weno::face_sum(P, cp, M, cm);
-    weno::derivative_plus(P, wp, cp, d + 8 * i);
-    weno::derivative_minus(M, wm, cm, d + 8 * i + 4);
+    const weno::Mean rp = P.mean_plus(wp), rm = M.mean_minus(wm);
+    sum[i] = weno::face_sum(P, rp, M, rm);
+    weno::derivative_plus(P, wp, rp, d + 8 * i);
+    weno::derivative_minus(M, wm, rm, d + 8 * i + 4);
   }
 }
 
