@@ -270,78 +270,71 @@ __global__ void __launch_bounds__(vlines_of(NV) * NV) k_adj_faces_lin(const doub
 }
 
 // Cell pass: cotangents of U, u_n and p of cell c from the per-position sums
-// of k_adj_faces, with the ghost positions that copy cell c folded back.
-// Returns via references.
+// of k_adj_faces, with the ghost positions that copy cell c folded back. Each
+// slot pair (dL/dF+, dL/dF-) is read by exactly one cell, which leaves it zero
+// for the next face pass.
+struct CellSums {
+  double a_un = 0.0, a_p = 0.0, a_alpha = 0.0;
+};
+
+// The pairs of position e along direction xdir of cell (i, j)'s line.
 template <int NV>
-__device__ __forceinline__ void gather_dir(const StateView& S, double* __restrict__ GF, const GridDev& g,
-                                           double ha, int xdir, int i, int j, double* aU, double& a_un, double& a_p,
-                                           double& a_alpha) {
-  const long long n = g.n;
+__device__ __forceinline__ void take_pairs(double* __restrict__ GF, const GridDev& g, int xdir, int i, int j, int e,
+                                           double2* f) {
   const int nx = g.nx, ny = g.ny;
-  const int ncell = xdir ? nx : ny;
-  const int c = xdir ? i : j;
-  const int line = xdir ? j : i;
-  const int bc_lo = xdir ? g.bc[0] : g.bc[2], bc_hi = xdir ? g.bc[1] : g.bc[3];
-  const int nmom = xdir ? 1 : 2;
-  const long long idx = (long long)j * nx + i;
-  const double un0 = S.plane(xdir ? NV + 1 : NV + 2, n)[idx];
-  const double hp = 0.5 * S.plane(NV + 3, n)[idx];
-  double Uc[NV];
+  double2* gf = reinterpret_cast<double2*>(GF) +
+                (xdir ? (long long)j * (nx + 6) + (e + 3) : (long long)(e + 3) * nx + i);
+  const long long kstride = xdir ? (long long)ny * (nx + 6) : (long long)(ny + 6) * nx;
 #pragma unroll
-  for (int k = 0; k < NV; ++k) Uc[k] = S.plane(k, n)[idx];
-  // positions that read cell c: c itself and the ghost images that map to it
-  int pos[7];
-  bool fl[7];
-  int np = 0;
-  pos[np] = c; fl[np++] = false;
-  for (int e = -3; e <= -1; ++e) {
-    bool flip;
-    if (ghost_src(e, ncell, bc_lo, bc_hi, flip) == c) { pos[np] = e; fl[np++] = flip; }
+  for (int k = 0; k < NV; ++k) f[k] = gf[k * kstride];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) gf[k * kstride] = make_double2(0.0, 0.0);
+}
+
+// F+- = lambda+- U (+ hp on the normal momentum, + hp u_n on the energy) at a
+// position that holds cell c or, with its normal components negated, its mirror image.
+template <int NV>
+__device__ __forceinline__ void add_position(const double2* f, const double* Uc, double un0, double hp, double ha,
+                                             bool flip, int nmom, double* aU, CellSums& s) {
+  const double un = flip ? -un0 : un0;
+  const double lp = fma(0.5, un, ha), lm = fma(0.5, un, -ha);
+  double aLp = 0.0, aLm = 0.0, a_hp = 0.0, a_hpu = 0.0;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    const bool neg = flip && k == nmom;
+    const double U = neg ? -Uc[k] : Uc[k];
+    const double fp = f[k].x, fm = f[k].y;
+    aU[k] = fma(neg ? -lp : lp, fp, fma(neg ? -lm : lm, fm, aU[k]));
+    aLp = fma(U, fp, aLp);
+    aLm = fma(U, fm, aLm);
+    if (k == nmom) a_hp += fp + fm;
+    if (k == 3) a_hpu += fp + fm;
   }
-  for (int e = ncell; e <= ncell + 2; ++e) {
+  const double a_un = 0.5 * (aLp + aLm) + hp * a_hpu;
+  s.a_alpha += 0.5 * (aLp - aLm);
+  s.a_p += 0.5 * (a_hp + un * a_hpu);
+  s.a_un += flip ? -a_un : a_un;
+}
+
+// The ghost images of a cell within three cells of a side.
+template <int NV>
+__device__ __forceinline__ void add_images(double* __restrict__ GF, const GridDev& g, int xdir, int i, int j,
+                                           const double* Uc, double un0, double hp, double ha, double* aU,
+                                           CellSums& s) {
+  const int ncell = xdir ? g.nx : g.ny, c = xdir ? i : j;
+  if (c >= 3 && c < ncell - 3) return;
+#pragma unroll 1
+  for (int t = 0; t < 6; ++t) {
+    const int e = t < 3 ? t - 3 : ncell + t - 3;
     bool flip;
-    if (ghost_src(e, ncell, bc_lo, bc_hi, flip) == c) { pos[np] = e; fl[np++] = flip; }
-  }
-  for (int t = 0; t < np; ++t) {
-    const int e = pos[t];
-    const bool flip = fl[t];
-    const double un = flip ? -un0 : un0;
-    const double lp = fma(0.5, un, ha), lm = fma(0.5, un, -ha);
-    double aLp = 0.0, aLm = 0.0, a_hp = 0.0, a_hpu = 0.0;
-    // all loads first, then the zeroing (each slot is read by exactly one
-    // cell: the sums are left zero for the next face pass), so the loads are
-    // not held behind the stores
-    double* gf0 = GF + 2 * (xdir ? ((long long)line) * (nx + 6) + (e + 3) : ((long long)(e + 3)) * nx + line);
-    const long long kstride = 2 * (xdir ? (long long)ny * (nx + 6) : (long long)(ny + 6) * nx);
-    double fpk[NV], fmk[NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      fpk[k] = gf0[k * kstride];
-      fmk[k] = gf0[k * kstride + 1];
-    }
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      gf0[k * kstride] = 0.0;
-      gf0[k * kstride + 1] = 0.0;
-    }
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      const double U = (flip && k == nmom) ? -Uc[k] : Uc[k];
-      const double fp = fpk[k], fm = fmk[k];
-      const double aUk = lp * fp + lm * fm;
-      aU[k] += (flip && k == nmom) ? -aUk : aUk;
-      aLp = fma(U, fp, aLp);
-      aLm = fma(U, fm, aLm);
-      if (k == nmom) a_hp += fp + fm;
-      if (k == 3) a_hpu += fp + fm;
-    }
-    // F+- = lambda+- U (+ hp on the normal momentum, + hp u_n on the energy)
-    const double a_un_e = 0.5 * (aLp + aLm) + hp * a_hpu;
-    a_alpha += 0.5 * (aLp - aLm);
-    a_p += 0.5 * (a_hp + un * a_hpu);
-    a_un += flip ? -a_un_e : a_un_e;
+    if (ghost_src(e, ncell, xdir ? g.bc[0] : g.bc[2], xdir ? g.bc[1] : g.bc[3], flip) != c) continue;
+    double2 f[NV];
+    take_pairs<NV>(GF, g, xdir, i, j, e, f);
+    add_position<NV>(f, Uc, un0, hp, ha, flip, xdir ? 1 : 2, aU, s);
   }
 }
+
+__device__ __forceinline__ void prefetch(const double* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
 // A mass-action monomial prod_s X_{sp(s)}^{a(s)} over n <= MAX_SIDE distinct
 // species (sp, a: accessors of the reaction side): the value, the gradient
@@ -382,6 +375,7 @@ __device__ __forceinline__ void monomial(const double* X, SP sp, A a, int n, con
     for (int t = 0; t < n; ++t) {
       double v;
       if (t == s) {
+        if (a(s) < 2) continue;
         v = P2[s];
 #pragma unroll
         for (int w = 0; w < n; ++w)
@@ -494,7 +488,7 @@ __device__ __forceinline__ void argmax_merge(unsigned long long& m, int& i, unsi
   if (m2 > m || (m2 == m && i2 < i)) { m = m2; i = i2; }
 }
 
-// Cell pass of the RHS VJP (256 threads per block). Besides the gathered
+// Cell pass of the RHS VJP (at most 128 threads per block, a power of two). Besides the gathered
 // cotangents it leaves, per block, the block sums of the alpha cotangents
 // (atomically added) and the arg-max of |u|+c and |v|+c over its cells in
 // part_mx / part_id [2 * block + direction].
@@ -502,7 +496,7 @@ __device__ __forceinline__ void argmax_merge(unsigned long long& m, int& i, unsi
 // source S(U) at this stage state, (dS/dU)^T mu (src_grad, with the rate
 // constants from src_keep when the forward kept them).
 template <int NS, bool SRC>
-__global__ void k_adj_cells(StateView S, const double* __restrict__ alpha2, double* __restrict__ GFx,
+__global__ void __launch_bounds__(128, NS <= 3 ? 5 : 3) k_adj_cells(StateView S, const double* __restrict__ alpha2, double* __restrict__ GFx,
                             double* __restrict__ GFy, VjpIO io, double* adj_alpha, GridDev g,
                             const MechDev* __restrict__ mech, unsigned long long* __restrict__ part_mx,
                             int* __restrict__ part_id, const double* __restrict__ src_keep) {
@@ -515,46 +509,60 @@ __global__ void k_adj_cells(StateView S, const double* __restrict__ alpha2, doub
   if (i < g.nx && j < g.ny) {
     const long long n = g.n;
     const long long idx = (long long)j * g.nx + i;
-    double aU[NV];
+    // every load of the cell is under way before the first is used
+    double u[NV], aU[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) aU[k] = 0.0;
-    double a_u = 0.0, a_v = 0.0, a_p = 0.0;
-    gather_dir<NV>(S, GFx, g, 0.5 * alpha2[0], 1, i, j, aU, a_u, a_p, ax);
-    gather_dir<NV>(S, GFy, g, 0.5 * alpha2[1], 0, i, j, aU, a_v, a_p, ay);
-    double u[NV];
+    for (int k = 0; k < NV; ++k) {
+      u[k] = S.plane(k, n)[idx];
+      aU[k] = 0.0;
+    }
+    const double T = S.plane(NV, n)[idx], un = S.plane(NV + 1, n)[idx], vn = S.plane(NV + 2, n)[idx];
+    const double hp = 0.5 * S.plane(NV + 3, n)[idx];
+    const double hax = 0.5 * alpha2[0], hay = 0.5 * alpha2[1];
+    double2 fx[NV], fy[NV];
+    take_pairs<NV>(GFx, g, 1, i, j, i, fx);
+    take_pairs<NV>(GFy, g, 0, i, j, j, fy);
 #pragma unroll
-    for (int k = 0; k < NV; ++k) u[k] = S.plane(k, n)[idx];
-    const double T = S.plane(NV, n)[idx];
+    for (int k = 0; k < NV; ++k) {
+      const long long kq = (long long)k * n + idx;
+      if (io.acc_a) prefetch(io.a + kq);
+      if (io.xa) prefetch(io.xa + kq);
+      if (io.b) prefetch(io.xb + kq);
+    }
+    CellSums sX, sY;
+    add_position<NV>(fx, u, un, hp, hax, false, 1, aU, sX);
+    add_images<NV>(GFx, g, 1, i, j, u, un, hp, hax, aU, sX);
+    add_position<NV>(fy, u, vn, hp, hay, false, 2, aU, sY);
+    add_images<NV>(GFy, g, 0, i, j, u, vn, hp, hay, aU, sY);
+    ax = sX.a_alpha;
+    ay = sY.a_alpha;
+    const double a_u = sX.a_un, a_v = sY.a_un, a_p = sX.a_p + sY.a_p;
     const double rrho = rcp(u[0]);
     const double vx = u[1] * rrho, vy = u[2] * rrho;
-    CellThermo<NS> ct;
-    cell_thermo<NS>(u, T, *mech, ct);
-    double dT[NV], dp[NV];
-    dT_dp_dU<NS>(u, T, *mech, ct, dT, dp);
+    const CellHeat ct = cell_heat<NS>(u, T, rrho, *mech);
     aU[0] += -(vx * a_u + vy * a_v) * rrho;
     aU[1] += a_u * rrho;
     aU[2] += a_v * rrho;
+    double a_T = 0.0;
     if constexpr (SRC) {
       constexpr int NSP = NS - 1;
       const MechDev& m = *mech;
       double w[NSP];
 #pragma unroll
       for (int k = 0; k < NSP; ++k) w[k] = m.M[k] * (io.mu_scale * io.lam[(long long)(4 + k) * n + idx]);
-      double gT, gX[NS];
-      src_grad<NS>(u, T, m, w, src_keep, n, idx, gT, gX);
+      double gX[NS];
+      src_grad<NS>(u, T, m, w, src_keep, n, idx, a_T, gX);
       const double gN = gX[NSP] * m.invM[NSP];
+      aU[0] += gN;
 #pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        double d = gT * dT[k];
-        if (k == 0) d += gN;
-        if (k >= 4) d += fma(gX[k - 4], m.invM[k - 4], -gN);
-        aU[k] += d;
-      }
+      for (int k = 0; k < NSP; ++k) aU[4 + k] += fma(gX[k], m.invM[k], -gN);
     }
+    const double s = RU * a_p;
+    add_thermo_grad<NS>(T, vx, vy, *mech, fma(s, ct.W, a_T) * rcp(ct.Cv), s * T, aU);
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
       const long long kq = (long long)k * n + idx;
-      double va = fma(dp[k], a_p, aU[k]);  // nu
+      double va = aU[k];  // nu
       if (io.acc_a) va += io.a[kq];
       if (io.xa) va = fma(io.ca, io.xa[kq], va);
       io.a[kq] = va;
@@ -564,16 +572,14 @@ __global__ void k_adj_cells(StateView S, const double* __restrict__ alpha2, doub
       }
     }
     // the LF speeds of this cell, as the forward's alpha max formed them
-    const double c = sound_speed<NS>(u, T, *mech);
-    const double rr = rcp(u[0]);
-    sx = dbits(dabs(u[1] * rr) + c);
-    sy = dbits(dabs(u[2] * rr) + c);
+    sx = dbits(dabs(vx) + ct.c);
+    sy = dbits(dabs(vy) + ct.c);
     cid = (int)idx;
   }
   // block sums of the alpha cotangents and block arg-max of the speeds
-  __shared__ double rx[256], ry[256];
-  __shared__ unsigned long long mx[2][256];
-  __shared__ int id[2][256];
+  __shared__ double rx[128], ry[128];
+  __shared__ unsigned long long mx[2][128];
+  __shared__ int id[2][128];
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
   rx[tid] = ax;
   ry[tid] = ay;
@@ -614,14 +620,20 @@ __global__ void k_adj_alpha(StateView S, GridDev g, const MechDev* __restrict__ 
   __shared__ unsigned long long mx[2][256];
   __shared__ int id[2][256];
   const int tid = threadIdx.x;
-#pragma unroll
-  for (int d = 0; d < 2; ++d) {
-    unsigned long long m = 0;
-    int i = 0x7fffffff;
-    for (int b = tid; b < nb; b += blockDim.x) argmax_merge(m, i, part_mx[2 * b + d], part_id[2 * b + d]);
-    mx[d][tid] = m;
-    id[d][tid] = i;
+  unsigned long long mX = 0, mY = 0;
+  int iX = 0x7fffffff, iY = 0x7fffffff;
+  // unrolled, so that four loads are in flight
+#pragma unroll 4
+  for (int b = tid; b < nb; b += blockDim.x) {
+    const ulonglong2 v = reinterpret_cast<const ulonglong2*>(part_mx)[b];
+    const int2 q = reinterpret_cast<const int2*>(part_id)[b];
+    argmax_merge(mX, iX, v.x, q.x);
+    argmax_merge(mY, iY, v.y, q.y);
   }
+  mx[0][tid] = mX;
+  id[0][tid] = iX;
+  mx[1][tid] = mY;
+  id[1][tid] = iY;
   __syncthreads();
   for (int s = blockDim.x / 2; s > 0; s >>= 1) {
     if (tid < s) {
@@ -647,18 +659,23 @@ __global__ void k_adj_alpha(StateView S, GridDev g, const MechDev* __restrict__ 
     for (int q = 0; q < NV; ++q) u[q] = S.plane(q, n)[cidx];
     const double T = S.plane(NV, n)[cidx];
     const MechDev& m = *mech;
-    CellThermo<NS> ct;
-    cell_thermo<NS>(u, T, m, ct);
-    const double rho = u[0];
-    // component k of dT/dU and dp/dU (as dT_dp_dU forms them)
-    const double rrho = 1.0 / rho;
+    const double rrho = rcp(u[0]);
+    const CellHeat ct = cell_heat<NS>(u, T, rrho, m);
+    // component k of dT/dU and dp/dU (as dT_dp_dU forms them): only the lane's
+    // own species and the last one are needed beside the mixture's sums
     const double vx = u[1] * rrho, vy = u[2] * rrho;
-    const double fN = (ct.hR[NS - 1] - T) * m.invM[NS - 1];
+    auto cv_R = [&](int q) {
+      const double* h = m.hc[q];
+      return fma(T, fma(T, fma(T, fma(T, 5.0 * h[4], 4.0 * h[3]), 3.0 * h[2]), 2.0 * h[1]), h[0]) - 1.0;
+    };
+    const int ks = k >= 4 ? k - 4 : NS - 1;  // the lane's species
+    const double fS = (enthalpy_R(m, ks, T) - T) * m.invM[ks], cS = cv_R(ks) * m.invM[ks];
+    const double fN = (enthalpy_R(m, NS - 1, T) - T) * m.invM[NS - 1], cN = cv_R(NS - 1) * m.invM[NS - 1];
     double dF, dWk = 0.0, dz_cv = 0.0;
     if (k == 0) {
       dF = fN - 0.5 * (vx * vx + vy * vy) * (1.0 / RU);
       dWk = m.invM[NS - 1];
-      dz_cv = ct.cvR[NS - 1] * m.invM[NS - 1];
+      dz_cv = cN;
     } else if (k == 1) {
       dF = vx * (1.0 / RU);
     } else if (k == 2) {
@@ -666,25 +683,23 @@ __global__ void k_adj_alpha(StateView S, GridDev g, const MechDev* __restrict__ 
     } else if (k == 3) {
       dF = -1.0 / RU;
     } else {
-      dF = (ct.hR[k - 4] - T) * m.invM[k - 4] - fN;
-      dWk = m.invM[k - 4] - m.invM[NS - 1];
-      dz_cv = ct.cvR[k - 4] * m.invM[k - 4] - ct.cvR[NS - 1] * m.invM[NS - 1];
+      dF = fS - fN;
+      dWk = m.invM[ks] - m.invM[NS - 1];
+      dz_cv = cS - cN;
     }
-    const double rCv = 1.0 / ct.Cv;
+    const double Cv = ct.Cv, Cp = ct.Cv + ct.W;
+    const double rCv = rcp(Cv);
     const double dTk = -dF * rCv;
     const double dpk = RU * (T * dWk + ct.W * dTk);
     const double p = RU * ct.W * T;
-    const double Cv = ct.Cv, Cp = ct.Cv + ct.W;
-    const double c = sqrt(Cp * p / (Cv * rho));
-    const double vel = u[1 + d] / rho;
+    const double vel = d ? vy : vx;
     const double sgn = vel < 0.0 ? -1.0 : 1.0;
     const double dCv = dz_cv + ct.dCv * dTk;
     const double dCp = dCv + dWk;
-    const double drho = k == 0 ? 1.0 : 0.0;
-    const double dc = 0.5 * c * (dCp / Cp + dpk / p - dCv / Cv - drho / rho);
+    const double dc = 0.5 * ct.c * (dCp * rcp(Cp) + dpk * rcp(p) - dCv * rCv - (k == 0 ? rrho : 0.0));
     double dvel = 0.0;
-    if (k == 0) dvel = -vel / rho;
-    if (k == 1 + d) dvel = 1.0 / rho;
+    if (k == 0) dvel = -vel * rrho;
+    if (k == 1 + d) dvel = rrho;
     contrib = a * (sgn * dvel + dc);
   }
   const double cy = __shfl_down_sync(0xffffffffu, contrib, 16);
@@ -793,6 +808,11 @@ __device__ __forceinline__ void chem_reverse_reactions(const MechDev& m, const d
                                                        const double* mu, double dt, const Cache& cache, double& gT_out,
                                                        double* gX) {
   constexpr int NSP = NS - 1;
+  // third bodies: coefficient one for every species, corrected for the few
+  // whose coefficient differs
+  double xtot = xe[0], vtot = 0.0;
+#pragma unroll
+  for (int k = 1; k < NS; ++k) xtot += xe[k];
   double gT = 0.0;
 #pragma unroll
   for (int k = 0; k < NS; ++k) gX[k] = 0.0;
@@ -816,10 +836,12 @@ __device__ __forceinline__ void chem_reverse_reactions(const MechDev& m, const d
     double Mi = 1.0, DMi = 0.0;
     if (R.tb()) {
       Mi = Ctot;
+      DMi = xtot;
 #pragma unroll
-      for (int e = 0; e < R.neff(); ++e) Mi = fma(m.effv[i][e], X[R.effsp(e)], Mi);
-#pragma unroll
-      for (int j = 0; j < NS; ++j) DMi = fma(1.0 + m.effm1[i][j], xe[j], DMi);
+      for (int e = 0; e < R.neff(); ++e) {
+        Mi = fma(m.effv[i][e], X[R.effsp(e)], Mi);
+        DMi = fma(m.effv[i][e], xe[R.effsp(e)], DMi);
+      }
     }
     const double MD = Mi + DMi;
     const double kfp = kf * cache.dk_f(R), kbp = kb * cache.dk_b(R);
@@ -836,10 +858,13 @@ __device__ __forceinline__ void chem_reverse_reactions(const MechDev& m, const d
     }
     if (R.tb()) {
       const double v = w * (net + Dnet);
+      vtot += v;
 #pragma unroll
-      for (int j = 0; j < NS; ++j) gX[j] = fma(1.0 + m.effm1[i][j], v, gX[j]);
+      for (int e = 0; e < R.neff(); ++e) gX[R.effsp(e)] = fma(m.effv[i][e], v, gX[R.effsp(e)]);
     }
   });
+#pragma unroll
+  for (int k = 0; k < NS; ++k) gX[k] += vtot;
   gT_out = gT;
 }
 
@@ -850,12 +875,11 @@ __device__ __forceinline__ void chem_vjp_out(const double* u, double T, const Me
                                              const double* gX, double* out) {
   constexpr int NSP = NS - 1;
   constexpr int NV = NS + 3;
-  CellThermo<NS> ct;
-  cell_thermo<NS>(u, T, m, ct);
-  double dT[NV], dp[NV];
-  dT_dp_dU<NS>(u, T, m, ct, dT, dp);
+  const double rrho = rcp(u[0]);
+  const double vx = u[1] * rrho, vy = u[2] * rrho;
 #pragma unroll
-  for (int q = 0; q < NV; ++q) out[q] = fma(gT, dT[q], lam[q]);
+  for (int q = 0; q < NV; ++q) out[q] = lam[q];
+  add_thermo_grad<NS>(T, vx, vy, m, gT * rcp(cell_heat<NS>(u, T, rrho, m).Cv), 0.0, out);
   const double gN = gX[NSP] * m.invM[NSP];
   out[0] += gN;
 #pragma unroll
@@ -1314,8 +1338,19 @@ __global__ void k_prim_T_vjp(const double* __restrict__ T, const double* __restr
 // ---------------------------------------------------------------------------
 static unsigned nblk(long long count, int thr) { return (unsigned)((count + thr - 1) / thr); }
 
-// Cell-pass blocks of 32 x 8 cells.
-static int adj_cell_blocks(const GridDev& g) { return ((g.nx + 31) / 32) * ((g.ny + 7) / 8); }
+// Cell-pass blocks of 32 x 4 cells while that gives at least 4 blocks per SM,
+// else 32 x 2 or 1, so that a small grid's cells spread over all SMs (512 x 64:
+// 62 us with 8 rows, 41 with 1).
+static int adj_cell_rows(const GridDev& g) {
+  const long long bxs = (g.nx + 31) / 32;
+  int by = 4;
+  while (by > 1 && bxs * ((g.ny + by - 1) / by) < 4LL * sm_count()) by /= 2;
+  return by;
+}
+static int adj_cell_blocks(const GridDev& g) {
+  const int by = adj_cell_rows(g);
+  return ((g.nx + 31) / 32) * ((g.ny + by - 1) / by);
+}
 
 size_t rhs_vjp_scratch_bytes(const GridDev& g) {
   return 256 + (((size_t)adj_cell_blocks(g) * 2 * (sizeof(unsigned long long) + sizeof(int)) + 255) & ~(size_t)255);
@@ -1358,7 +1393,8 @@ static cudaError_t rhs_vjp_t(const StateView& S, const double* alpha2_dev, const
     if (lin) k_adj_faces_lin<NV, 8><<<total, VLINES * NV, 0, st>>>(lin, mu, ms, CFx, CFy, g, nbx, ntx_x, ntx_y);
     else k_adj_faces<NV, 8><<<total, VLINES * NV, 0, st>>>(S, alpha2_dev, mu, ms, CFx, CFy, g, nbx, ntx_x, ntx_y);
   }
-  dim3 blk(32, 8), grd((g.nx + 31) / 32, (g.ny + 7) / 8);
+  const int by = adj_cell_rows(g);
+  dim3 blk(32, by), grd((g.nx + 31) / 32, (g.ny + by - 1) / by);
   bool done = false;
   if constexpr (NS > 1) {
     if (src) {

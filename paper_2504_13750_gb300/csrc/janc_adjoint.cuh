@@ -71,4 +71,45 @@ __device__ __forceinline__ void dT_dp_dU(const double* u, double T, const MechDe
   }
 }
 
+// W, Cv = sum z_k cv_k / Ru and dCv/dT of one cell at T, on the mixture sums
+// of the forward (janc_device.cuh), and the frozen sound speed as sound_speed
+// forms it.
+struct CellHeat {
+  double W, Cv, dCv, c;
+};
+template <int NS>
+__device__ __forceinline__ CellHeat cell_heat(const double* u, double T, double rrho, const MechDev& m) {
+  CellHeat r;
+  double h[5];
+  mixture_sums<NS, 5>(u, m, r.W, h);
+  const double c1 = 2.0 * h[1], c2 = 3.0 * h[2], c3 = 4.0 * h[3], c4 = 5.0 * h[4];
+  r.Cv = fma(T, fma(T, fma(T, fma(T, c4, c3), c2), c1), h[0] - r.W);
+  r.dCv = fma(T, fma(T, fma(T, 4.0 * c4, 3.0 * c3), 2.0 * c2), c1);
+  r.c = speed(r.Cv + r.W, RU * r.W * T, rrho, r.Cv);
+  return r;
+}
+
+__device__ __forceinline__ double enthalpy_R(const MechDev& m, int k, double T) {
+  const double* h = m.hc[k];
+  return fma(T, fma(T, fma(T, fma(T, fma(T, h[4], h[3]), h[2]), h[1]), h[0]), h[5]);
+}
+
+// a += sW dW/dU - sF dF/dU: the chain through T(U) and p = Ru W T (dT_dp_dU)
+// with the two scalars formed first, sF = (Ru W a_p + a_T) / Cv and sW = Ru T a_p
+// for cotangents a_T and a_p. 9 FP64 instructions a species; with the species'
+// own cv, dT/dU and dp/dU it took 24.
+template <int NS>
+__device__ __forceinline__ void add_thermo_grad(double T, double vx, double vy, const MechDev& m, double sF, double sW,
+                                                double* a) {
+  const double q = sF * (1.0 / RU);
+  const double fN = (enthalpy_R(m, NS - 1, T) - T) * m.invM[NS - 1];
+  a[0] = fma(-sF, fN, fma(0.5 * q, fma(vx, vx, vy * vy), fma(sW, m.invM[NS - 1], a[0])));
+  a[1] = fma(-q, vx, a[1]);
+  a[2] = fma(-q, vy, a[2]);
+  a[3] += q;
+#pragma unroll
+  for (int k = 0; k < NS - 1; ++k)
+    a[4 + k] = fma(-sF, fma(enthalpy_R(m, k, T) - T, m.invM[k], -fN), fma(sW, m.Wd[k], a[4 + k]));
+}
+
 }  // namespace janc
