@@ -738,6 +738,7 @@ __global__ void k_adj_alpha(StateView S, GridDev g, const MechDev* __restrict__ 
 // shared memory (one column of 4 NR doubles per thread, every index a
 // constant) for the compiled structure.
 struct LocalRateCache {
+  static constexpr bool kScaled = false;
   double kf[MAX_NR], kb[MAX_NR], dkf[MAX_NR], dkb[MAX_NR];
   __device__ __forceinline__ void put(int i, double a, double b, double c, double d) {
     kf[i] = a; kb[i] = b; dkf[i] = c; dkb[i] = d;
@@ -750,6 +751,7 @@ struct LocalRateCache {
   __device__ __forceinline__ double dk_b(const Rx& R) const { return dkb[R.idx()]; }
 };
 struct SharedRateCache {
+  static constexpr bool kScaled = false;
   double* col;  // this thread's column: entry q at col[q * stride]
   int stride;
   __device__ __forceinline__ void put(int i, double a, double b, double c, double d) {
@@ -766,12 +768,13 @@ struct SharedRateCache {
   __device__ __forceinline__ double dk_b(const Rx& R) const { return col[(4 * R.idx() + 3) * stride]; }
 };
 // The rate constants the segment recompute's chemistry kept (k_chem_lin:
-// k_f, k_b of reaction i at entries 2i, 2i+1 of cell q) and their log-T
+// dt k_f, dt k_b of reaction i at entries 2i, 2i+1 of cell q) and their log-T
 // derivatives formed here, as the forward pass of chem_vjp_rev forms them:
 // d ln k_f/dT = b/T + Ea/(R T^2), d ln k_b/dT = d ln k_f/dT + sum over the
 // reactants of dG - sum over the products of dG + dnu/T.
 template <int NS>
 struct StoredRateCache {
+  static constexpr bool kScaled = true;  // k_f and k_b come with the factor dt
   const double* clin;
   long long n, q;
   double rT, rT2;
@@ -826,7 +829,7 @@ __device__ __forceinline__ void chem_reverse_reactions(const MechDev& m, const d
 #pragma unroll
     for (int r = 0; r < npr; ++r)
       if (R.psp(r) < NSP) mi = fma(R.pnud(r), mu[R.psp(r)], mi);
-    const double w = dt * mi;
+    const double w = Cache::kScaled ? mi : dt * mi;
     const double kf = cache.k_f(i), kb = cache.k_b(i);
     double F, gF[MAX_SIDE], DF, hF[MAX_SIDE], B, gB[MAX_SIDE], DB, hB[MAX_SIDE];
     monomial(X, [&](int s_) { return R.rsp(s_); }, [&](int s_) { return R.rnu(s_); }, nre, xe, F, gF, DF, hF);

@@ -171,10 +171,10 @@ __global__ void __launch_bounds__(AB2) k_amr_update(StateView Sin, StateView S0,
                                                     unsigned long long* alpha_out, int* status) {
   constexpr int NV = NS + 3;
   const double dt = step_dt(ctl, a_step);  // the layer's dt: fixed, or from the base layer's LF speeds
-  const int blk = blockIdx.x;
-  const int i = threadIdx.x % AB, j = threadIdx.x / AB;
   const long long n = L.n;
-  const long long idx = (long long)blk * AB2 + j * AB + i;
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int blk = (int)(idx / AB2), cell = (int)(idx % AB2);
+  const int i = cell % AB, j = cell / AB;
   double u[NV];
   double T, p, c, rrho;
   int st = 0;
@@ -560,14 +560,25 @@ GridDev layer_grid(const janc_amr_s* A, int i) {  // for the per-cell chemistry 
   return g;
 }
 
+// Threads per block of the kernels with a thread per cell: the 256 cells of an
+// AMR block while that gives at least 4 blocks per SM, else 128, 64 or 32, so
+// that a few refined blocks spread over all SMs (59 AMR blocks: an update takes
+// 22.6 us in blocks of 256, 16 in blocks of 32).
+int cell_threads(long long cells) {
+  int t = AB2;
+  while (t > 32 && (cells + t - 1) / t < 4LL * sm_count()) t /= 2;
+  return t;
+}
+
 cudaError_t launch_alpha(int ns, const StateView& S, long long n, const MechDev* mech, unsigned long long* out,
                          int* status, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)((n + 255) / 256);
+  const int t = cell_threads(n);
+  const unsigned blocks = (unsigned)((n + t - 1) / t);
   switch (ns) {
-    case 1: k_amr_alpha<1><<<blocks, 256, 0, st>>>(S, n, mech, out, status); break;
-    case 3: k_amr_alpha<3><<<blocks, 256, 0, st>>>(S, n, mech, out, status); break;
-    case 9: k_amr_alpha<9><<<blocks, 256, 0, st>>>(S, n, mech, out, status); break;
+    case 1: k_amr_alpha<1><<<blocks, t, 0, st>>>(S, n, mech, out, status); break;
+    case 3: k_amr_alpha<3><<<blocks, t, 0, st>>>(S, n, mech, out, status); break;
+    case 9: k_amr_alpha<9><<<blocks, t, 0, st>>>(S, n, mech, out, status); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -590,6 +601,7 @@ cudaError_t solve_layer_t(janc_amr_s* A, int i, const StepCtl& lc) {
   if (e == cudaSuccess) e = launch_alpha(NS, S0, D.n, gp.mech, a, A->d_status, st);
   const size_t smem = sizeof(double) * (NV + 4) * ALINES * AWIN;
   const unsigned ftiles = 4u * (unsigned)L.nblk;
+  const int ut = cell_threads(D.n);
   const StateView ins[3] = {S0, S1, S2};
   const StateView outs[3] = {S1, S2, S0};
   for (int s = 0; s < 3 && e == cudaSuccess; ++s) {
@@ -597,13 +609,13 @@ cudaError_t solve_layer_t(janc_amr_s* A, int i, const StepCtl& lc) {
     e = cudaGetLastError();
     if (e != cudaSuccess) break;
     if (s == 0)
-      k_amr_update<NS, 1><<<L.nblk, AB2, 0, st>>>(ins[s], S0, outs[s], L.Fx, L.Gy, D, P, gp.mech, lc, gp.alpha, a + 2,
+      k_amr_update<NS, 1><<<L.nblk * (AB2 / ut), ut, 0, st>>>(ins[s], S0, outs[s], L.Fx, L.Gy, D, P, gp.mech, lc, gp.alpha, a + 2,
                                                   A->d_status);
     else if (s == 1)
-      k_amr_update<NS, 2><<<L.nblk, AB2, 0, st>>>(ins[s], S0, outs[s], L.Fx, L.Gy, D, P, gp.mech, lc, gp.alpha, a + 4,
+      k_amr_update<NS, 2><<<L.nblk * (AB2 / ut), ut, 0, st>>>(ins[s], S0, outs[s], L.Fx, L.Gy, D, P, gp.mech, lc, gp.alpha, a + 4,
                                                   A->d_status);
     else
-      k_amr_update<NS, 3><<<L.nblk, AB2, 0, st>>>(ins[s], S0, outs[s], L.Fx, L.Gy, D, P, gp.mech, lc, gp.alpha, a + 6,
+      k_amr_update<NS, 3><<<L.nblk * (AB2 / ut), ut, 0, st>>>(ins[s], S0, outs[s], L.Fx, L.Gy, D, P, gp.mech, lc, gp.alpha, a + 6,
                                                   A->d_status);
     e = cudaGetLastError();
   }

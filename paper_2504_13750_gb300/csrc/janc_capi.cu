@@ -93,6 +93,53 @@ int check_desc(const janc_grid_desc* d, const janc_mechanism* m) {
   return JANC_OK;
 }
 
+// The fixed-point tables of the rate constants (MechDev::gq, kq).
+void fixed_rate_table(MechDev* h) {
+  const double log2e = 1.4426950408889634074;
+  bool ok = true;
+  auto fix = [&](double v, int bits, double limit) {
+    if (!(std::fabs(v) < limit)) ok = false;
+    return ok ? (long long)std::nearbyint(std::ldexp(v, bits)) : 0ll;
+  };
+  for (int k = 0; k < h->ns; ++k) {
+    const double* c = h->gc[k];
+    h->gq[k][0] = fix(c[0], 58, 31.0);
+    double sum = 0.0;
+    for (int q = 1; q < 5; ++q) {
+      const double v = std::ldexp(c[q] * log2e, 13 * q);
+      h->gq[k][q] = fix(v, 54, 200.0);
+      sum += std::fabs(v);
+    }
+    if (!(sum < 500.0)) ok = false;
+    h->gq[k][5] = fix(c[5] * log2e, 46, 65535.0);
+    h->gq[k][6] = fix(c[6] * log2e, 54, 500.0);
+  }
+  for (int i = 0; i < h->nr; ++i) {
+    h->kq[i][0] = fix(h->lnA[i] * log2e, 54, 500.0);
+    h->kq[i][1] = fix(h->b[i], 58, 31.0);
+    h->kq[i][2] = fix(-h->EaR[i] * log2e, 46, 65535.0);
+  }
+  h->lref = fix(std::log2(RU / P_REF), 54, 500.0);
+  // the logarithms are smooth in ln T: 241 points leave nothing between them
+  // that could reach from 440 to the 512 the arithmetic holds less the 70 of dt
+  for (int s = 0; ok && s <= 240; ++s) {
+    const double T = 256.0 * std::pow(2.0, 5.0 * s / 240.0), lnT = std::log(T);
+    double G[MAX_NS];
+    for (int k = 0; k < h->ns; ++k) {
+      const double* c = h->gc[k];
+      G[k] = c[0] * lnT + c[6] + T * (c[1] + T * (c[2] + T * (c[3] + T * c[4]))) + c[5] / T;
+    }
+    for (int i = 0; i < h->nr; ++i) {
+      const double f = h->lnA[i] + h->b[i] * lnT - h->EaR[i] / T;
+      double b = f + h->dnu[i] * std::log(RU / P_REF * T);
+      for (int r = 0; r < h->nre[i]; ++r) b += h->rnu[i][r] * G[h->rsp[i][r]];
+      for (int r = 0; r < h->npr[i]; ++r) b -= h->pnu[i][r] * G[h->psp[i][r]];
+      if (!(std::fabs(f) * log2e < 430.0 && std::fabs(b) * log2e < 430.0)) ok = false;
+    }
+  }
+  h->rate_ok = ok;
+}
+
 int build_mech(const janc_mechanism* m, MechDev* h) {
   std::memset(h, 0, sizeof(MechDev));
   const int ns = m->ns;
@@ -113,6 +160,7 @@ int build_mech(const janc_mechanism* m, MechDev* h) {
     h->gc[k][5] = -a[5];
     h->gc[k][6] = a[6] - a[0];
     h->mratio[k] = m->M[k] / m->M[ns - 1];
+    h->third[k] = 1.0 - h->mratio[k];
   }
   h->WN = h->invM[ns - 1];
   for (int q = 0; q < 6; ++q) h->hcN[q] = h->hc[ns - 1][q] * h->invM[ns - 1];
@@ -185,6 +233,7 @@ int build_mech(const janc_mechanism* m, MechDev* h) {
       h->ceff[i][l] = el - h->mratio[l] * eN;
     }
   }
+  fixed_rate_table(h);
   return JANC_OK;
 }
 

@@ -14,11 +14,6 @@
 // compares and selects. Then Newton T for the new state, aux planes and the
 // alpha max for the next step.
 //
-// exp(G_k) is formed once per species so that each reverse rate costs a few
-// multiplications instead of a second exponential per reaction; the
-// exponentials use the table-driven exp_t (about half the FP64 instructions
-// of the library exp).
-//
 // The reaction loop is written once over a structure policy: DynRx reads each
 // reaction's species, coefficients and third-body data from the run-time
 // table, FixRx<I> returns them as compile-time constants of the shipped H2-air
@@ -39,10 +34,89 @@ namespace janc {
 
 constexpr int CHEM_THREADS = 128;
 
+// G_k of Eq. 4.9.
+__device__ __forceinline__ double gibbs(const MechDev& m, int k, double T, double lnT, double rT) {
+  const double* c = m.gc[k];
+  return fma(c[0], lnT, fma(c[5], rT, fma(T, fma(T, fma(T, fma(T, c[4], c[3]), c[2]), c[1]), c[6])));
+}
+
+// c0 log2 T + c5 / T + c6 in units of 2^-54 for T = 2^e (1 + ..) in [256, 8192): L =
+// log2 T in units of 2^-60, y = 2^(64 + e) / T; the factors as in MechDev::kq.
+__device__ __forceinline__ long long fixed_arrhenius(long long c6, long long c0, long long c5, soft::u64 L, soft::u64 y,
+                                                     int e) {
+  return c6 + soft::mulhi_signed(L, c0) + soft::sar(soft::mulhi_signed(y, c5), e - 8);
+}
+
+// dt k_f and dt k_b of every reaction of the compiled structure, at
+// out[2 i stride] and out[(2 i + 1) stride], from their base-2 logarithms in fixed
+// point, units of 2^-54. log2 k_b is log2 k_f plus integer sums of the G_k, and
+// dt and the power of P_ref/(Ru T) are summands, so that a reaction takes two
+// exponentials, 2 x 55 integer instructions, and no FP64 one. (As FP64
+// polynomials, nine exp(G_k), their reciprocals and products it was 196 of the
+// cell's 1080 FP64 instructions.) The logarithms are good to about 2^-51; as
+// doubles, at sizes of 30 to 100, the G_k are good to 2^-48. The sums may wrap on
+// the way, the results are within +-512 (MechDev::rate_ok). Cells outside
+// 256 K <= T < 8192 K, time steps outside 2^-70 .. 2^20 and tables that do not fit
+// take the FP64 form.
+template <int NS>
+__device__ __forceinline__ void rate_constants(const MechDev& m, double T, double dt, double* __restrict__ out,
+                                               int stride) {
+  using namespace soft;
+  constexpr int NR = fixed_h2air::NR;
+  const Parts t(T), d(dt);
+  if (m.rate_ok && !t.neg && t.e >= 1031 && t.e < 1036 && !d.neg && d.e > 953 && d.e < 1043) {
+    const int e = t.e - 1023;
+    const u64 L = ((u64)e << 60) + (log2_frac(t.m) >> 4);
+    const u64 y = recip_normal(t.m);
+    const u64 x = shr(t.m, 12 - e);  // T / 8192
+    const long long ldt = ((long long)(d.e - 1023) << 54) + (long long)(log2_frac(d.m) >> 10);
+    const long long lref = m.lref + (long long)(L >> 6);
+    long long G[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      const long long* c = m.gq[k];
+      long long p = mulhi_signed(x, c[4]);
+#pragma unroll
+      for (int q = 3; q > 0; --q) p = mulhi_signed(x, c[q] + p);
+      G[k] = p + fixed_arrhenius(c[6], c[0], c[5], L, y, e);
+    }
+    for_reactions<true>(m, [&](auto R) {
+      const int i = R.idx();
+      const long long f = fixed_arrhenius(m.kq[i][0] + ldt, m.kq[i][1], m.kq[i][2], L, y, e);
+      long long b = f + R.dnu() * lref;
+#pragma unroll
+      for (int r = 0; r < R.nre(); ++r) b += R.rnu(r) * G[R.rsp(r)];
+#pragma unroll
+      for (int r = 0; r < R.npr(); ++r) b -= R.pnu(r) * G[R.psp(r)];
+      out[(2 * i) * stride] = __longlong_as_double(f);
+      out[(2 * i + 1) * stride] = __longlong_as_double(b);
+    });
+    // in a loop: 38 copies of the code in line wait for their instructions
+#pragma unroll 1
+    for (int i = 0; i < NR; ++i) {
+#pragma unroll
+      for (int q = 2 * i; q < 2 * i + 2; ++q) out[q * stride] = exp2_fixed(__double_as_longlong(out[q * stride]));
+    }
+  } else {
+    const double lnT = log_t(T), rT = rcp(T), lcr = log_t((RU / P_REF) * T);
+#pragma unroll 1
+    for (int i = 0; i < NR; ++i) {
+      const double f = fma(m.b[i], lnT, fma(-m.EaR[i], rT, m.lnA[i]));
+      double b = fma((double)m.dnu[i], lcr, f);
+#pragma unroll 1
+      for (int r = 0; r < m.nre[i]; ++r) b = fma(m.rnud[i][r], gibbs(m, m.rsp[i][r], T, lnT, rT), b);
+#pragma unroll 1
+      for (int r = 0; r < m.npr[i]; ++r) b = fma(-m.pnud[i][r], gibbs(m, m.psp[i][r], T, lnT, rT), b);
+      out[(2 * i) * stride] = dt * exp_t(f);
+      out[(2 * i + 1) * stride] = dt * exp_t(b);
+    }
+  }
+}
+
 // One CHEM_THREADS block `blk` of cells; shared by the single-grid and the
 // batched kernels. STORE (the discrete adjoint's segment recompute): also
 // keep, per cell, what the chemistry VJP reuses (chem_lin_entries doubles,
-// entry e of cell q at clin[e * n + q]): k_f and k_b of every reaction
+// entry e of cell q at clin[e * n + q]): dt k_f and dt k_b of every reaction
 // (2i, 2i+1), then at 2 nr the LU factors of A = I - dt J'' in elimination
 // order (row r, column k at 2 nr + r (ns-1) + k: the multiplier of row r at
 // elimination step k for r > k, U for r < k, 1/U_kk on the diagonal), the
@@ -52,6 +126,10 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
                                            const StepCtl& ctl, const unsigned long long* __restrict__ alpha_step,
                                            unsigned long long* alpha_out, int* status, long long blk,
                                            double* __restrict__ clin = nullptr) {
+  // FIXED: the thread's column of rate constants
+  const int exs = blockDim.x;
+  extern __shared__ double ex_cols[];
+  double* const ex = ex_cols + threadIdx.x;
   constexpr int NSP = NS - 1;
   constexpr int NV = NS + 3;
   const MechDev& m = *mech;
@@ -79,25 +157,30 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
 #pragma unroll
     for (int k = 1; k < NS; ++k) Ctot += X[k];
 
-    const double lnT = log_t(T);
-    const double rT = rcp(T);
-    // exp(G_k) and exp(-G_k), G_k = s_k/R - h_k/(RT) (Eq. 4.9 bracket)
+    const double lnT = FIXED ? 0.0 : log_t(T);
+    const double rT = FIXED ? 0.0 : rcp(T);
+    // dt k_f and dt k_b (ex, 2 i and 2 i + 1) with the compiled structure; for a
+    // run-time table exp(G_k) and exp(-G_k), G_k = s_k/R - h_k/(RT) (Eq. 4.9 bracket)
     double eG[NS], reG[NS];
+    if constexpr (FIXED) {
+      rate_constants<NS>(m, T, dt, ex, exs);
+    } else {
 #pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      const double* c = m.gc[k];
-      const double G = fma(c[0], lnT, fma(c[5], rT, fma(T, fma(T, fma(T, fma(T, c[4], c[3]), c[2]), c[1]), c[6])));
-      eG[k] = exp_t(G);
-      reG[k] = rcp(eG[k]);
+      for (int k = 0; k < NS; ++k) {
+        eG[k] = exp_t(gibbs(m, k, T, lnT, rT));
+        reG[k] = rcp(eG[k]);
+      }
     }
     const double cref = (P_REF / RU) * rT;   // P_ref / (Ru T)
     const double rcref = (RU / P_REF) * T;
 
-    double wd[NSP];        // molar production rates of the carried species
-    double J[NSP][NSP];    // J'' of the header comment
+    // everything from k_f on carries the factor dt
+    double wd[NSP];        // dt x molar production rates of the carried species
+    double J[NSP][NSP];    // dt J'' of the header comment, less the third bodies' common part
+    double S3[NSP];        // that part: row k is S3[k] (1 - M_l / M_ns)
 #pragma unroll
     for (int k = 0; k < NSP; ++k) {
-      wd[k] = 0.0;
+      wd[k] = S3[k] = 0.0;
 #pragma unroll
       for (int l = 0; l < NSP; ++l) J[k][l] = 0.0;
     }
@@ -105,49 +188,84 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
     for_reactions<FIXED>(m, [&](auto R) {
       const int i = R.idx();
       const int nre = R.nre(), npr = R.npr();
-      const double kf = exp_t(fma(m.b[i], lnT, fma(-m.EaR[i], rT, m.lnA[i])));
-      // k_b = k_f / K_eq,  K_eq = prod_j exp(G_j)^{nu_j} (P_ref/(Ru T))^{dnu}
-      double kb = kf;
-#pragma unroll
-      for (int r = 0; r < nre; ++r)
-#pragma unroll
-        for (int q = 0; q < R.rnu(r); ++q) kb *= eG[R.rsp(r)];
-#pragma unroll
-      for (int r = 0; r < npr; ++r)
-#pragma unroll
-        for (int q = 0; q < R.pnu(r); ++q) kb *= reG[R.psp(r)];
-      const int dn = R.dnu();
-#pragma unroll
-      for (int q = 0; q < dn; ++q) kb *= rcref;
-#pragma unroll
-      for (int q = 0; q < -dn; ++q) kb *= cref;
+      double kf, kb;
+      if constexpr (FIXED) {
+        kf = ex[(2 * i) * exs];
+        kb = ex[(2 * i + 1) * exs];
+      } else {
+        kf = kb = dt * exp_t(fma(m.b[i], lnT, fma(-m.EaR[i], rT, m.lnA[i])));
+        // k_b = k_f / K_eq,  K_eq = prod_j exp(G_j)^{nu_j} (P_ref/(Ru T))^{dnu}
+        for (int r = 0; r < nre; ++r)
+          for (int q = 0; q < R.rnu(r); ++q) kb *= eG[R.rsp(r)];
+        for (int r = 0; r < npr; ++r)
+          for (int q = 0; q < R.pnu(r); ++q) kb *= reG[R.psp(r)];
+        const int dn = R.dnu();
+        for (int q = 0; q < dn; ++q) kb *= rcref;
+        for (int q = 0; q < -dn; ++q) kb *= cref;
+      }
       if (STORE) {
         clin[(2LL * i) * n + idx] = kf;
         clin[(2LL * i + 1) * n + idx] = kb;
       }
-      // law of mass action and its derivatives with respect to each participant
-      double xr[MAX_SIDE], xp[MAX_SIDE];
-      double fwd = kf, bwd = kb;
+      // law of mass action and its derivatives with respect to each
+      // participant; a rate is its first derivative times that concentration
+      double xr[MAX_SIDE], xp[MAX_SIDE], dq[2 * MAX_SIDE];
+      int dsp[2 * MAX_SIDE];
+#pragma unroll
+      for (int r = 0; r < nre; ++r) xr[r] = X[R.rsp(r)];
+#pragma unroll
+      for (int r = 0; r < npr; ++r) xp[r] = X[R.psp(r)];
 #pragma unroll
       for (int r = 0; r < nre; ++r) {
-        xr[r] = X[R.rsp(r)];
+        double d = R.rnu(r) == 1 ? kf : kf * R.rnud(r);
 #pragma unroll
-        for (int q = 0; q < R.rnu(r); ++q) fwd *= xr[r];
+        for (int s = 0; s < nre; ++s) {
+          const int pw = R.rnu(s) - (s == r ? 1 : 0);
+#pragma unroll
+          for (int t = 0; t < pw; ++t) d *= xr[s];
+        }
+        dq[r] = d;
+        dsp[r] = R.rsp(r);
       }
 #pragma unroll
       for (int r = 0; r < npr; ++r) {
-        xp[r] = X[R.psp(r)];
+        double d = R.pnu(r) == 1 ? kb : kb * R.pnud(r);
 #pragma unroll
-        for (int q = 0; q < R.pnu(r); ++q) bwd *= xp[r];
+        for (int s = 0; s < npr; ++s) {
+          const int pw = R.pnu(s) - (s == r ? 1 : 0);
+#pragma unroll
+          for (int t = 0; t < pw; ++t) d *= xp[s];
+        }
+        dq[nre + r] = -d;
+        dsp[nre + r] = R.psp(r);
       }
-      double Mi = 1.0;
-      if (R.tb()) {
-        Mi = Ctot;
+      double fwd = kf, bwd = kb;
+      if (R.rnu(0) == 1) {
+        fwd = dq[0] * xr[0];
+      } else {
 #pragma unroll
-        for (int e = 0; e < R.neff(); ++e) Mi = fma(m.effv[i][e], X[R.effsp(e)], Mi);
+        for (int r = 0; r < nre; ++r)
+#pragma unroll
+          for (int q = 0; q < R.rnu(r); ++q) fwd *= xr[r];
+      }
+      if (R.pnu(0) == 1) {
+        bwd = -dq[nre] * xp[0];
+      } else {
+#pragma unroll
+        for (int r = 0; r < npr; ++r)
+#pragma unroll
+          for (int q = 0; q < R.pnu(r); ++q) bwd *= xp[r];
       }
       const double net = fwd - bwd;
-      const double q = Mi * net;
+      double q = net;
+      if (R.tb()) {
+        double Mi = Ctot;
+#pragma unroll
+        for (int e = 0; e < R.neff(); ++e) Mi = fma(m.effv[i][e], X[R.effsp(e)], Mi);
+        q = Mi * net;
+#pragma unroll
+        for (int d = 0; d < nre + npr; ++d) dq[d] *= Mi;
+      }
       // sources: wdot_k += nu_ki q
 #pragma unroll
       for (int r = 0; r < nre; ++r) {
@@ -159,35 +277,14 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
         const int k = R.psp(r);
         if (k < NSP) wd[k] = fma(R.pnud(r), q, wd[k]);
       }
-      // dq/dX_j for the participants (third-body factor held fixed here)
-      double dq[2 * MAX_SIDE];
-      int dsp[2 * MAX_SIDE];
-      int nd = 0;
+      // rows: every carried species with nonzero net coefficient. A third-body
+      // coefficient of one in every column goes to S3; one of the last species
+      // that differs from one changes all columns.
+      bool last = false;
+      if (R.tb()) {
 #pragma unroll
-      for (int r = 0; r < nre; ++r) {
-        double d = R.rnu(r) == 1 ? kf : kf * R.rnud(r);
-#pragma unroll
-        for (int s = 0; s < nre; ++s) {
-          const int pw = R.rnu(s) - (s == r ? 1 : 0);
-#pragma unroll
-          for (int t = 0; t < pw; ++t) d *= xr[s];
-        }
-        dq[nd] = Mi * d;
-        dsp[nd++] = R.rsp(r);
+        for (int e = 0; e < R.neff(); ++e) last = last || R.effsp(e) == NSP;
       }
-#pragma unroll
-      for (int r = 0; r < npr; ++r) {
-        double d = R.pnu(r) == 1 ? kb : kb * R.pnud(r);
-#pragma unroll
-        for (int s = 0; s < npr; ++s) {
-          const int pw = R.pnu(s) - (s == r ? 1 : 0);
-#pragma unroll
-          for (int t = 0; t < pw; ++t) d *= xp[s];
-        }
-        dq[nd] = -Mi * d;
-        dsp[nd++] = R.psp(r);
-      }
-      // rows: every carried species with nonzero net coefficient
 #pragma unroll
       for (int side = 0; side < 2; ++side) {
         const int cnt = side ? npr : nre;
@@ -209,8 +306,14 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
           }
           if (R.tb()) {
             const double v = nu * net;
+            if (last) {
 #pragma unroll
-            for (int l = 0; l < NSP; ++l) J[k][l] = fma(v, m.ceff[i][l], J[k][l]);
+              for (int l = 0; l < NSP; ++l) J[k][l] = fma(v, m.ceff[i][l], J[k][l]);
+            } else {
+              S3[k] += v;
+#pragma unroll
+              for (int e = 0; e < R.neff(); ++e) J[k][R.effsp(e)] = fma(v, m.effv[i][e], J[k][R.effsp(e)]);
+            }
           }
         }
       }
@@ -220,9 +323,12 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
     double A[NSP][NSP], b[NSP], ip[NSP];
 #pragma unroll
     for (int k = 0; k < NSP; ++k) {
-      b[k] = dt * wd[k];
+      b[k] = wd[k];
 #pragma unroll
-      for (int l = 0; l < NSP; ++l) A[k][l] = fma(-dt, J[k][l], k == l ? 1.0 : 0.0);
+      for (int l = 0; l < NSP; ++l) {
+        A[k][l] = fma(-S3[k], m.third[l], -J[k][l]);
+        if (k == l) A[k][l] += 1.0;
+      }
     }
     bool singular = false;
     const long long lu0 = 2LL * m.nr;  // STORE: first LU entry
@@ -240,6 +346,7 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
       // the pivot row row c's old ones (nothing moves when piv == c). Written
       // as one gather and one scatter per column so that every index stays a
       // constant and the matrix stays in registers.
+      if (piv != c) {
 #pragma unroll
       for (int k = c; k < NSP; ++k) {
         const double ac = A[c][k];
@@ -258,6 +365,7 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
 #pragma unroll
         for (int r = c + 1; r < NSP; ++r) b[r] = (piv == r) ? bc : b[r];
         b[c] = v;
+      }
       }
       if (best == 0ull) singular = true;
       ip[c] = rcp(A[c][c]);
@@ -356,6 +464,9 @@ bool fixed_structure(const janc_mechanism* m) {
   return true;
 }
 
+// Shared memory of the compiled-structure kernels: k_f and k_b of every reaction.
+static size_t chem_smem(int threads) { return sizeof(double) * 2 * fixed_h2air::NR * threads; }
+
 cudaError_t launch_chem_batch(int ns, const BatchReq* reqs, const int* first, int nreq, int total, bool fixed,
                               cudaStream_t st) {
   const int sms = sm_count();
@@ -364,7 +475,7 @@ cudaError_t launch_chem_batch(int ns, const BatchReq* reqs, const int* first, in
   switch (ns) {
     case 3: k_chem_batch<3, false><<<grid, CHEM_THREADS, 0, st>>>(reqs, first, nreq); break;
     case 9:
-      if (fixed) k_chem_batch<9, true><<<grid, CHEM_THREADS, 0, st>>>(reqs, first, nreq);
+      if (fixed) k_chem_batch<9, true><<<grid, CHEM_THREADS, chem_smem(CHEM_THREADS), st>>>(reqs, first, nreq);
       else k_chem_batch<9, false><<<grid, CHEM_THREADS, 0, st>>>(reqs, first, nreq);
       break;
     default: return cudaErrorInvalidValue;
@@ -393,7 +504,7 @@ cudaError_t launch_chem(int ns, const StateView& S, const GridDev& g, const Mech
   switch (ns) {
     case 3: k_chem<3, false><<<blocks, thr, 0, st>>>(S, g, mech, ctl, alpha_step, alpha_out, status); break;
     case 9:
-      if (g.chem_fixed) k_chem<9, true><<<blocks, thr, 0, st>>>(S, g, mech, ctl, alpha_step, alpha_out, status);
+      if (g.chem_fixed) k_chem<9, true><<<blocks, thr, chem_smem(thr), st>>>(S, g, mech, ctl, alpha_step, alpha_out, status);
       else k_chem<9, false><<<blocks, thr, 0, st>>>(S, g, mech, ctl, alpha_step, alpha_out, status);
       break;
     default: return cudaErrorInvalidValue;
@@ -412,7 +523,7 @@ cudaError_t launch_chem_lin(int ns, const StateView& S, const GridDev& g, const 
     case 3: k_chem_lin<3, false><<<blocks, thr, 0, st>>>(S, g, mech, ctl, alpha_step, alpha_out, status, clin); break;
     case 9:
       if (g.chem_fixed)
-        k_chem_lin<9, true><<<blocks, thr, 0, st>>>(S, g, mech, ctl, alpha_step, alpha_out, status, clin);
+        k_chem_lin<9, true><<<blocks, thr, chem_smem(thr), st>>>(S, g, mech, ctl, alpha_step, alpha_out, status, clin);
       else
         k_chem_lin<9, false><<<blocks, thr, 0, st>>>(S, g, mech, ctl, alpha_step, alpha_out, status, clin);
       break;

@@ -60,6 +60,7 @@ struct MechDev {
   // eff_il - (M_l / M_ns) eff_i,ns for l < ns - 1.
   double ceff[MAX_NR][MAX_NS];
   double mratio[MAX_NS];  // M_l / M_ns
+  double third[MAX_NS];   // 1 - M_l / M_ns: ceff of a reaction whose coefficients are all one
   // Mixture sums in the carried variables: since rho Y_ns = rho - sum_{k<ns-1}
   // rho Y_k, sum_k (rho Y_k / M_k) c_k = rho cN + sum_{k<ns-1} rho Y_k cd_k
   // with cN = c_ns / M_ns and cd_k = c_k / M_k - cN. For the enthalpy
@@ -77,6 +78,13 @@ struct MechDev {
   unsigned mixs[7][MAX_NS];
   int mixe[7], mixp[MAX_NS];
   int mix_ok;  // every mixe within +-400
+  // G_k and ln k_f as base-2 logarithms in fixed point (fixed_rates): gq in the
+  // order of gc, the factor of log2 T in units of 2^-58, those of (T / 8192)^m and
+  // the constant of 2^-54, that of 1/T of 2^-46; kq: ln A, b, -Ea/R likewise;
+  // lref = log2(Ru / P_ref) in units of 2^-54. rate_ok: the numbers fit, and every
+  // log2 k_f and log2 k_b stays within +-440 for T in [256, 8192).
+  long long gq[MAX_NS][7], kq[MAX_NR][3], lref;
+  int rate_ok;
 };
 
 // Grid constants passed by value to every kernel.

@@ -265,6 +265,11 @@ JANC_HD u64 log2_frac(u64 m) {
   return JANC_LDG(&kLog2[j]) + (mulhi(l, 0xb8aa3b295c17f0bcull) >> 4);     // log2 e in units of 2^-63
 }
 
+// a b / 2^64 for signed b, at most 3 below the exact quotient.
+JANC_HD long long mulhi_signed(u64 a, long long b) {
+  return (long long)(mulhi(a, (u64)b) - (b < 0 ? a : 0ull));
+}
+
 // |x| = m 2^(e - 1086) with m in [2^63, 2^64), for a normal double.
 struct Parts {
   u64 m;
@@ -309,6 +314,9 @@ JANC_HD double exp_double(double x) {
   }
   return round_double(exp2_frac(a << 10), k);
 }
+
+// 2^(a 2^-54), within 0.6 units in the last place.
+JANC_HD double exp2_fixed(long long a) { return round_double(exp2_frac((u64)a << 10), (int)(a >> 54)); }
 
 // ln x for x in [2, 2^1023), within 2^-53 before the rounding to nearest.
 JANC_HD double log_double(double x) {

@@ -139,11 +139,6 @@ struct Weights {
   }
 };
 
-// u q / 2^64 for signed q, at most 3 below the exact quotient.
-JANC_HD long long mulhi_signed(u64 u, long long q) {
-  return (long long)(mulhi(u, (u64)q) - (q < 0 ? u : 0ull));
-}
-
 // The weighted mean r = n y of the substencils' offsets (Q_k / 6): Q_k as
 // integers in units of 2^(e_k - 1080) below 7 2^58, 3 2^58, 5 2^58. Their
 // products with the weights are aligned to the largest and summed below 2^63.
