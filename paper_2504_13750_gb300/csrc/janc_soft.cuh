@@ -287,6 +287,31 @@ JANC_HD double round_double(u64 m, int e) {
   return double_of((m >> 11) + ((m >> 10) & 1) + ((u64)(u32)((1022 + e) << 20) << 32));
 }
 
+// x cut to a float, 0 below a float's normal range; no check above it. And a
+// float as a double (2^-127 for 0). (The conversion instructions occupy the FP64 pipe.)
+JANC_HD float cut_float(double x) {
+  const u64 b = bits_of(x);
+  const u32 a = hi32(b) & 0x7fffffffu, n = a - 0x38000000u;
+  u32 f = (n << 3 | lo32(b) >> 29) | (hi32(b) & 0x80000000u);
+  if (a < 0x38100000u) f = 0;
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(f);
+#else
+  float r;
+  memcpy(&r, &f, 4);
+  return r;
+#endif
+}
+JANC_HD double widen(float x) {
+#ifdef __CUDA_ARCH__
+  const u32 f = __float_as_uint(x);
+#else
+  u32 f;
+  memcpy(&f, &x, 4);
+#endif
+  return double_of(((u64)((((f & 0x7fffffffu) >> 3) + 0x38000000u) | (f & 0x80000000u)) << 32) | (u64)(f << 29));
+}
+
 // 1/x for normal x of either sign, correctly rounded but for near ties; 0
 // beyond 2^1021, NaN for 0, denormals, infinities and NaN.
 JANC_HD double rcp_double(double x) {
