@@ -5,8 +5,8 @@
 //
 // One launch covers both directions: blocks [0, nbx) take x-face tiles and the
 // rest take y-face tiles. A tile is lines_of(NV) grid lines (rows for x, columns for
-// y) by 32 consecutive faces along them (16 or 8 on grids too small to fill
-// the GPU with 32-face tiles; the batched launch always uses 32). Its cells,
+// y) by 32 consecutive faces along them (16, 8 or 4 on grids too small to fill
+// the GPU with longer tiles; the batched launch always uses 32). Its cells,
 // with the 5-cell stencil
 // margin, are staged in shared memory once; every thread then owns one
 // (line, variable) and slides two 5-point windows (F+ and F-) along its line,
@@ -237,18 +237,22 @@ static cudaError_t launch_face_flux_fc(const StateView& S, const unsigned long l
   return cudaGetLastError();
 }
 
-// Tile length by grid size: 32 faces while that gives at least 8 blocks per
-// SM, 16 while that gives at least 2, else 8. Shorter tiles mean more blocks
-// and a larger share of stencil margin; on small grids, whose launches are a
-// fraction of a wave and latency-bound, the blocks win (measured on one
-// GB300: 256 x 32 runs best at 8, 512 x 64 at 16, 4096 x 512 at 32).
+// Tile length by grid size: 32 faces while that gives at least 24 warps per SM,
+// 16 while that gives at least 6, 8 while that gives at least 3, else 4. Shorter
+// tiles mean more blocks and a larger share of stencil margin; on small grids,
+// whose launches are a fraction of a wave and latency-bound, the blocks win
+// (128 x 16, 12 variables: 12.9 us with 8, 8.6 with 4; 256 x 32 runs best at 8, 512 x 64
+// at 16, 4096 x 512 at 32). Four variables are one warp a block: 1021 x 257 takes
+// 106 us with 32 and 85 with 16.
 static int flux_tile_faces(const GridDev& g, int nv) {
-  const int sms = sm_count();
+  const int sms = sm_count(), warps = (lines_of(nv) * nv + 31) / 32;
   int nbx, ntx_x, ntx_y, total;
   tiles_of(g, nv, 32, &nbx, &ntx_x, &ntx_y, &total);
-  if (total >= 8 * sms) return 32;
+  if (total * warps >= 24 * sms) return 32;
   tiles_of(g, nv, 16, &nbx, &ntx_x, &ntx_y, &total);
-  return total >= 2 * sms ? 16 : 8;
+  if (total * warps >= 6 * sms) return 16;
+  tiles_of(g, nv, 8, &nbx, &ntx_x, &ntx_y, &total);
+  return total * warps >= 3 * sms ? 8 : 4;
 }
 
 template <int NV, bool HALO>
@@ -257,7 +261,8 @@ static cudaError_t launch_face_flux_h(const StateView& S, const unsigned long lo
   switch (flux_tile_faces(g, NV)) {
     case 32: return launch_face_flux_fc<NV, 32, HALO>(S, alpha, Fx, Gy, g, st);
     case 16: return launch_face_flux_fc<NV, 16, HALO>(S, alpha, Fx, Gy, g, st);
-    default: return launch_face_flux_fc<NV, 8, HALO>(S, alpha, Fx, Gy, g, st);
+    case 8: return launch_face_flux_fc<NV, 8, HALO>(S, alpha, Fx, Gy, g, st);
+    default: return launch_face_flux_fc<NV, 4, HALO>(S, alpha, Fx, Gy, g, st);
   }
 }
 
@@ -288,7 +293,8 @@ static cudaError_t launch_face_flux_lin_t(const StateView& S, const unsigned lon
   switch (flux_tile_faces(g, NV)) {
     case 32: return launch_face_flux_lin_fc<NV, 32>(S, alpha, Fx, Gy, lin, g, st);
     case 16: return launch_face_flux_lin_fc<NV, 16>(S, alpha, Fx, Gy, lin, g, st);
-    default: return launch_face_flux_lin_fc<NV, 8>(S, alpha, Fx, Gy, lin, g, st);
+    case 8: return launch_face_flux_lin_fc<NV, 8>(S, alpha, Fx, Gy, lin, g, st);
+    default: return launch_face_flux_lin_fc<NV, 4>(S, alpha, Fx, Gy, lin, g, st);
   }
 }
 
