@@ -34,19 +34,6 @@ namespace janc {
 
 constexpr int CHEM_THREADS = 128;
 
-// G_k of Eq. 4.9.
-__device__ __forceinline__ double gibbs(const MechDev& m, int k, double T, double lnT, double rT) {
-  const double* c = m.gc[k];
-  return fma(c[0], lnT, fma(c[5], rT, fma(T, fma(T, fma(T, fma(T, c[4], c[3]), c[2]), c[1]), c[6])));
-}
-
-// c0 log2 T + c5 / T + c6 in units of 2^-54 for T = 2^e (1 + ..) in [256, 8192): L =
-// log2 T in units of 2^-60, y = 2^(64 + e) / T; the factors as in MechDev::kq.
-__device__ __forceinline__ long long fixed_arrhenius(long long c6, long long c0, long long c5, soft::u64 L, soft::u64 y,
-                                                     int e) {
-  return c6 + soft::mulhi_signed(L, c0) + soft::sar(soft::mulhi_signed(y, c5), e - 8);
-}
-
 // dt k_f and dt k_b of every reaction of the compiled structure, at
 // out[2 i stride] and out[(2 i + 1) stride], from their base-2 logarithms in fixed
 // point, units of 2^-54. log2 k_b is log2 k_f plus integer sums of the G_k, and
@@ -63,27 +50,17 @@ __device__ __forceinline__ void rate_constants(const MechDev& m, double T, doubl
                                                int stride) {
   using namespace soft;
   constexpr int NR = fixed_h2air::NR;
-  const Parts t(T), d(dt);
-  if (m.rate_ok && !t.neg && t.e >= 1031 && t.e < 1036 && !d.neg && d.e > 953 && d.e < 1043) {
-    const int e = t.e - 1023;
-    const u64 L = ((u64)e << 60) + (log2_frac(t.m) >> 4);
-    const u64 y = recip_normal(t.m);
-    const u64 x = shr(t.m, 12 - e);  // T / 8192
+  const Parts d(dt);
+  FixedT t;
+  if (fixed_T(m, T, t) && !d.neg && d.e > 953 && d.e < 1043) {
     const long long ldt = ((long long)(d.e - 1023) << 54) + (long long)(log2_frac(d.m) >> 10);
-    const long long lref = m.lref + (long long)(L >> 6);
     long long G[NS];
 #pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      const long long* c = m.gq[k];
-      long long p = mulhi_signed(x, c[4]);
-#pragma unroll
-      for (int q = 3; q > 0; --q) p = mulhi_signed(x, c[q] + p);
-      G[k] = p + fixed_arrhenius(c[6], c[0], c[5], L, y, e);
-    }
+    for (int k = 0; k < NS; ++k) G[k] = fixed_gibbs(m, k, t);
     for_reactions<true>(m, [&](auto R) {
       const int i = R.idx();
-      const long long f = fixed_arrhenius(m.kq[i][0] + ldt, m.kq[i][1], m.kq[i][2], L, y, e);
-      long long b = f + R.dnu() * lref;
+      const long long f = fixed_arrhenius(m.kq[i][0] + ldt, m.kq[i][1], m.kq[i][2], t);
+      long long b = f + R.dnu() * t.lref;
 #pragma unroll
       for (int r = 0; r < R.nre(); ++r) b += R.rnu(r) * G[R.rsp(r)];
 #pragma unroll
@@ -101,12 +78,8 @@ __device__ __forceinline__ void rate_constants(const MechDev& m, double T, doubl
     const double lnT = log_t(T), rT = rcp(T), lcr = log_t((RU / P_REF) * T);
 #pragma unroll 1
     for (int i = 0; i < NR; ++i) {
-      const double f = fma(m.b[i], lnT, fma(-m.EaR[i], rT, m.lnA[i]));
-      double b = fma((double)m.dnu[i], lcr, f);
-#pragma unroll 1
-      for (int r = 0; r < m.nre[i]; ++r) b = fma(m.rnud[i][r], gibbs(m, m.rsp[i][r], T, lnT, rT), b);
-#pragma unroll 1
-      for (int r = 0; r < m.npr[i]; ++r) b = fma(-m.pnud[i][r], gibbs(m, m.psp[i][r], T, lnT, rT), b);
+      double f, b;
+      log_rates(m, i, T, lnT, rT, lcr, f, b);
       out[(2 * i) * stride] = dt * exp_t(f);
       out[(2 * i + 1) * stride] = dt * exp_t(b);
     }

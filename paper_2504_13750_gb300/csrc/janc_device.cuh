@@ -270,6 +270,54 @@ __device__ __forceinline__ double sound_speed(const double* u, double t, const M
   return speed(Cp, p, rrho, Cv);
 }
 
+// G_k of Eq. 4.9.
+__device__ __forceinline__ double gibbs(const MechDev& m, int k, double T, double lnT, double rT) {
+  const double* c = m.gc[k];
+  return fma(c[0], lnT, fma(c[5], rT, fma(T, fma(T, fma(T, fma(T, c[4], c[3]), c[2]), c[1]), c[6])));
+}
+
+// T in [256, 8192) = 2^e (1 + ..) for the fixed-point logarithms of the rate
+// constants: L = log2 T in units of 2^-60, y = 2^(64 + e) / T, x = T / 8192 in units
+// of 2^-64, lref = log2(Ru T / P_ref) in units of 2^-54. False where T is outside
+// or the mechanism's numbers do not fit (MechDev::rate_ok).
+struct FixedT {
+  soft::u64 L, y, x;
+  int e;
+  long long lref;
+};
+__device__ __forceinline__ bool fixed_T(const MechDev& m, double T, FixedT& t) {
+  const soft::Parts p(T);
+  if (!m.rate_ok || p.neg || p.e < 1031 || p.e >= 1036) return false;
+  t.e = p.e - 1023;
+  t.L = ((soft::u64)t.e << 60) + (soft::log2_frac(p.m) >> 4);
+  t.y = soft::recip_normal(p.m);
+  t.x = soft::shr(p.m, 12 - t.e);
+  t.lref = m.lref + (long long)(t.L >> 6);
+  return true;
+}
+// c0 log2 T + c5 / T + c6 in units of 2^-54, the factors as in MechDev::kq.
+__device__ __forceinline__ long long fixed_arrhenius(long long c6, long long c0, long long c5, const FixedT& t) {
+  return c6 + soft::mulhi_signed(t.L, c0) + soft::sar(soft::mulhi_signed(t.y, c5), t.e - 8);
+}
+// G_k log2 e in units of 2^-54.
+__device__ __forceinline__ long long fixed_gibbs(const MechDev& m, int k, const FixedT& t) {
+  const long long* c = m.gq[k];
+  long long p = soft::mulhi_signed(t.x, c[4]);
+#pragma unroll
+  for (int q = 3; q > 0; --q) p = soft::mulhi_signed(t.x, c[q] + p);
+  return p + fixed_arrhenius(c[6], c[0], c[5], t);
+}
+// ln k_f and ln k_b of reaction i in FP64, lcr = ln(Ru T / P_ref).
+__device__ __forceinline__ void log_rates(const MechDev& m, int i, double T, double lnT, double rT, double lcr,
+                                          double& f, double& b) {
+  f = fma(m.b[i], lnT, fma(-m.EaR[i], rT, m.lnA[i]));
+  b = fma((double)m.dnu[i], lcr, f);
+#pragma unroll 1
+  for (int r = 0; r < m.nre[i]; ++r) b = fma(m.rnud[i][r], gibbs(m, m.rsp[i][r], T, lnT, rT), b);
+#pragma unroll 1
+  for (int r = 0; r < m.npr[i]; ++r) b = fma(-m.pnud[i][r], gibbs(m, m.psp[i][r], T, lnT, rT), b);
+}
+
 // Molar production rates (Eq. 4.7-4.9) of the carried species k < ns - 1 at
 // (T, X(u)), for the explicit source-term form of the step.
 template <int NS>
@@ -291,27 +339,34 @@ __device__ __forceinline__ void carried_rates(const double* u, double T, const M
   double Ctot = X[0];
 #pragma unroll
   for (int k = 1; k < NS; ++k) Ctot += X[k];
-  const double lnT = log_t(T);
-  const double rT = rcp(T);
-  double eG[NS], reG[NS];
+  // the rate constants from their logarithms: fixed point, else FP64
+  FixedT t;
+  const bool fixed = fixed_T(m, T, t);
+  long long G[NS];
+  double lnT = 0.0, rT = 0.0, lcr = 0.0;
+  if (fixed) {
 #pragma unroll
-  for (int k = 0; k < NS; ++k) {
-    const double* c = m.gc[k];
-    eG[k] = exp_t(fma(c[0], lnT, fma(c[5], rT, fma(T, fma(T, fma(T, fma(T, c[4], c[3]), c[2]), c[1]), c[6]))));
-    reG[k] = rcp(eG[k]);
+    for (int k = 0; k < NS; ++k) G[k] = fixed_gibbs(m, k, t);
+  } else {
+    lnT = log_t(T);
+    rT = rcp(T);
+    lcr = log_t((RU / P_REF) * T);
   }
-  const double cref = (P_REF / RU) * rT;
-  const double rcref = (RU / P_REF) * T;
   for (int i = 0; i < m.nr; ++i) {
     const int nre = m.nre[i], npr = m.npr[i];
-    const double kf = exp_t(fma(m.b[i], lnT, fma(-m.EaR[i], rT, m.lnA[i])));
-    double kb = kf;
-    for (int r = 0; r < nre; ++r)
-      for (int q = 0; q < m.rnu[i][r]; ++q) kb *= eG[m.rsp[i][r]];
-    for (int r = 0; r < npr; ++r)
-      for (int q = 0; q < m.pnu[i][r]; ++q) kb *= reG[m.psp[i][r]];
-    for (int q = 0; q < m.dnu[i]; ++q) kb *= rcref;
-    for (int q = 0; q < -m.dnu[i]; ++q) kb *= cref;
+    double kf, kb;
+    if (fixed) {
+      const long long f = fixed_arrhenius(m.kq[i][0], m.kq[i][1], m.kq[i][2], t);
+      long long b = f + m.dnu[i] * t.lref;
+      for (int r = 0; r < nre; ++r) b += m.rnu[i][r] * G[m.rsp[i][r]];
+      for (int r = 0; r < npr; ++r) b -= m.pnu[i][r] * G[m.psp[i][r]];
+      kf = soft::exp2_fixed(f);
+      kb = soft::exp2_fixed(b);
+    } else {
+      log_rates(m, i, T, lnT, rT, lcr, kf, kb);
+      kf = exp_t(kf);
+      kb = exp_t(kb);
+    }
     if (keep) {
       keep[(2LL * i) * n + idx] = kf;
       keep[(2LL * i + 1) * n + idx] = kb;
