@@ -142,18 +142,24 @@ struct Weights {
 // The weighted mean r = n y of the substencils' offsets (Q_k / 6): Q_k as
 // integers in units of 2^(e_k - 1080) below 7 2^58, 3 2^58, 5 2^58. Their
 // products with the weights are aligned to the largest and summed below 2^63.
-// Not finite where a difference was not.
+// Not finite where a difference was not. s, t: the sum and its exponent,
+// r = s y 2^(t + x - 1149) with y and x of the weights.
 struct Mean {
   double n, y;
+  long long s;
+  int t;
+  bool bad;
   JANC_HD Mean(const Weights& w, long long q0, int e0, long long q1, int e1, long long q2, int e2) {
     const int t0 = e0 - 2 * w.d0, t1 = e1 - 2 * w.d1 + 2, t2 = e2 - 2 * w.d2 + 1;  // weights 1, 4 (1.5), 2 (1.5)
-    int t = t0 > t1 ? t0 : t1;
+    t = t0 > t1 ? t0 : t1;
     t = t > t2 ? t : t2;
     const long long v = sar(mulhi_signed(w.u1, q1), t - t1) + sar(mulhi_signed(w.u2, q2), t - t2);
-    n = scaled_double(sar(mulhi_signed(w.u0, q0), t - t0) + v + (v >> 1), t + w.x - 1085);
+    s = sar(mulhi_signed(w.u0, q0), t - t0) + v + (v >> 1);
+    n = scaled_double(s, t + w.x - 1085);
     int e = e0 > e1 ? e0 : e1;
     e = e > e2 ? e : e2;
-    if (e > 2000) n = double_of(0x7ff8000000000000ull);
+    bad = e > 2000;
+    if (bad) n = double_of(0x7ff8000000000000ull);
     y = round_double(w.y, -1);
   }
 };
@@ -232,8 +238,28 @@ JANC_HD double face_sum(const Win& P, const Mean& p, const Win& M, const Mean& m
 // w_k / C_k comes from the products of the weights and one more reciprocal,
 // that of C_0 C_1 C_2. (a_k, b_k): the pair of substencil k, first difference
 // first, in units of 2^(e_k - 1080): Q_k and dC_k/dd_m are small integer
-// combinations of them, formed on integers and converted, so that 14 FP64
-// instructions are left of 30.
+// combinations of them, and h_k is formed on integers too, so that six FP64
+// instructions are left of 30 (1000 x 400, 6 variables: 0.51 ms a launch, 0.56 with
+// h_k as doubles, 1.05 with all of it).
+
+// 2 (w_k / C_k) 6 (r - q_k) = g (6 r - Q_k) 2^x, g 2^64 at least 2^55: 6 r = v
+// 2^(ev - 1080), Q_k = q 2^(e - 1080), aligned to the larger.
+JANC_HD double weighted_gap(u64 g, int x, long long v, int ev, long long q, int e) {
+  const int top = ev > e ? ev : e;
+  const long long d = sar(v, top - ev) - sar(q, top - e);
+  u64 m = d < 0 ? 0ull - (u64)d : (u64)d;
+  x += top - 1080;
+  if (hi32(m) == 0) {
+    m <<= 32;
+    x -= 32;
+  }
+  int z = leading_zeros(hi32(m));  // 158 for 0
+  const u64 p = mulhi(g, shl(m, z));
+  const int f = 1085 + x - z;
+  z = leading_zeros(hi32(p));
+  const u64 b = (shl(p, z) >> 11) + ((u64)((u32)(f - z) << 20 | (hi32((u64)d) & 0x80000000u)) << 32);
+  return double_of(f - z < 0 || p == 0 ? 0ull : b);
+}
 JANC_HD void derivative(const Num& s0, const Num& s1, const Num& s2, const Weights& w, const Coef& c, const Mean& r,
                         long long a0, long long b0, int e0, long long a1, long long b1, int e1, long long a2,
                         long long b2, int e2, double* g) {
@@ -241,16 +267,16 @@ JANC_HD void derivative(const Num& s0, const Num& s1, const Num& s2, const Weigh
   const u64 y = recip(mulhi(w.p12, s0.n), &z);
   // 1 / C_0 = mulhi(p12, y) 2^(z - 127 + 2103 - e_0); twice the sixth of the weight over C_k
   const int b = w.x + z + 1 - 127 + 2103;
-  const double G0 = to_double(mulhi(c.u0, mulhi(w.p12, y)), b - 5 - 2 * w.d0 - s0.e + 64);
-  const double G1 = to_double(3 * (mulhi(c.u1, mulhi(w.p02, y)) >> 2), b - 2 - 2 * w.d1 - s1.e + 64);
-  const double G2 = to_double(3 * (mulhi(c.u2, mulhi(w.p01, y)) >> 2), b - 3 - 2 * w.d2 - s2.e + 64);
-  const double r6 = mul_rn(mul_rn(6.0, r.n), r.y);
+  const long long ri = mulhi_signed(w.y, r.s);
+  const long long v = (ri + (ri >> 1)) >> 1;  // 6 r in units of 2^(ev - 1080), below 2^62
+  const int ev = r.t + w.x - 2;
+  double h0 = weighted_gap(mulhi(c.u0, mulhi(w.p12, y)), b - 5 - 2 * w.d0 - s0.e + 64, v, ev, 5 * b0 - 2 * a0, e0);
+  double h1 = weighted_gap(3 * (mulhi(c.u1, mulhi(w.p02, y)) >> 2), b - 2 - 2 * w.d1 - s1.e + 64, v, ev, a1 + 2 * b1, e1);
+  double h2 = weighted_gap(3 * (mulhi(c.u2, mulhi(w.p01, y)) >> 2), b - 3 - 2 * w.d2 - s2.e + 64, v, ev, 4 * a2 - b2, e2);
+  if (r.bad) h0 = h1 = h2 = double_of(0x7ff8000000000000ull);
   e0 -= 1080;
   e1 -= 1080;
   e2 -= 1080;
-  const double h0 = G0 * sub_rn(r6, scaled_double(5 * b0 - 2 * a0, e0));
-  const double h1 = G1 * sub_rn(r6, scaled_double(a1 + 2 * b1, e1));
-  const double h2 = G2 * sub_rn(r6, scaled_double(4 * a2 - b2, e2));
   g[0] = fma(h0, scaled_double(8 * a0 - 11 * b0, e0), -c.k1);
   g[1] = fma(h1, scaled_double(8 * a1 - 5 * b1, e1), fma(h0, scaled_double(20 * b0 - 11 * a0, e0), c.k2));
   g[2] = fma(h2, scaled_double(20 * a2 - 11 * b2, e2), fma(h1, scaled_double(8 * b1 - 5 * a1, e1), c.k3));
