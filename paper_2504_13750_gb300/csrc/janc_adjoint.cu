@@ -151,7 +151,7 @@ __device__ __forceinline__ double* gf_base(const VjpTile& T, double* GFx, double
 }
 
 template <int NV, int VFACES>
-__global__ void __launch_bounds__(vlines_of(NV) * NV) k_adj_faces(StateView S, const double* __restrict__ alpha2,
+__global__ void __launch_bounds__(vlines_of(NV) * NV, 384 / (vlines_of(NV) * NV)) k_adj_faces(StateView S, const double* __restrict__ alpha2,
                                                            const double* __restrict__ mu, double mu_scale,
                                                            double* __restrict__ GFx, double* __restrict__ GFy,
                                                            GridDev g, int nbx, int ntx_x, int ntx_y) {

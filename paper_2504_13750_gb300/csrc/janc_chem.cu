@@ -393,16 +393,28 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
   block_reduce_alpha_status(sx, sy, st, alpha_out, status);
 }
 
-template <int NS, bool FIXED>
-__global__ void __launch_bounds__(CHEM_THREADS) k_chem(StateView S, GridDev g, const MechDev* __restrict__ mech,
+// BLOCKS of the compiled-structure kernels: 3 blocks of 128 threads an SM (12
+// warps) at 168 registers, of which 480 B spill, or no bound (230 registers, 8
+// warps). A third warp on each scheduler hides more than the spills cost (two steps
+// of 4096 x 512: 20.6 ms with 8, 19.4 with 12), but a full round of 12 takes 86 us
+// where one of 8 takes 74, so the sum of the rounds decides. A step of reactors, us
+// with 8 and with 12: 512 x 96 (10.1 warps an SM) 153 and 112, 512 x 128 (13.5) 154
+// and 153, 640 x 128 (16.8) 223 and 177, 2048 x 256 1033 and 872.
+static int chem_blocks_per_sm(long long n) {
+  const long long per = 32LL * sm_count(), w = (n + per - 1) / per;  // warps an SM gets
+  return 86 * ((w + 11) / 12) < 74 * ((w + 7) / 8) ? 3 : 0;
+}
+
+template <int NS, bool FIXED, int BLOCKS = 0>
+__global__ void __launch_bounds__(CHEM_THREADS, BLOCKS) k_chem(StateView S, GridDev g, const MechDev* __restrict__ mech,
                                                        StepCtl ctl, const unsigned long long* __restrict__ alpha_step,
                                                        unsigned long long* alpha_out, int* status) {
   chem_block<NS, FIXED>(S, g, mech, ctl, alpha_step, alpha_out, status, blockIdx.x);
 }
 
 // k_chem that also keeps the chemistry VJP's factors (chem_block, STORE).
-template <int NS, bool FIXED>
-__global__ void __launch_bounds__(CHEM_THREADS) k_chem_lin(StateView S, GridDev g, const MechDev* __restrict__ mech,
+template <int NS, bool FIXED, int BLOCKS = 0>
+__global__ void __launch_bounds__(CHEM_THREADS, BLOCKS) k_chem_lin(StateView S, GridDev g, const MechDev* __restrict__ mech,
                                                            StepCtl ctl,
                                                            const unsigned long long* __restrict__ alpha_step,
                                                            unsigned long long* alpha_out, int* status,
@@ -413,7 +425,7 @@ __global__ void __launch_bounds__(CHEM_THREADS) k_chem_lin(StateView S, GridDev 
 // Batched chemistry over the flattened (request, block) list: in place on
 // each request's S[0], output alpha in slot 4.
 template <int NS, bool FIXED>
-__global__ void __launch_bounds__(CHEM_THREADS) k_chem_batch(const BatchReq* __restrict__ reqs,
+__global__ void __launch_bounds__(CHEM_THREADS, FIXED ? 3 : 0) k_chem_batch(const BatchReq* __restrict__ reqs,
                                                              const int* __restrict__ first, int nreq) {
   const int total = first[nreq];
   for (int e = blockIdx.x; e < total; e += gridDim.x) {
@@ -477,7 +489,10 @@ cudaError_t launch_chem(int ns, const StateView& S, const GridDev& g, const Mech
   switch (ns) {
     case 3: k_chem<3, false><<<blocks, thr, 0, st>>>(S, g, mech, ctl, alpha_step, alpha_out, status); break;
     case 9:
-      if (g.chem_fixed) k_chem<9, true><<<blocks, thr, chem_smem(thr), st>>>(S, g, mech, ctl, alpha_step, alpha_out, status);
+      if (g.chem_fixed && chem_blocks_per_sm(g.n) == 3)
+        k_chem<9, true, 3><<<blocks, thr, chem_smem(thr), st>>>(S, g, mech, ctl, alpha_step, alpha_out, status);
+      else if (g.chem_fixed)
+        k_chem<9, true><<<blocks, thr, chem_smem(thr), st>>>(S, g, mech, ctl, alpha_step, alpha_out, status);
       else k_chem<9, false><<<blocks, thr, 0, st>>>(S, g, mech, ctl, alpha_step, alpha_out, status);
       break;
     default: return cudaErrorInvalidValue;
@@ -495,7 +510,9 @@ cudaError_t launch_chem_lin(int ns, const StateView& S, const GridDev& g, const 
   switch (ns) {
     case 3: k_chem_lin<3, false><<<blocks, thr, 0, st>>>(S, g, mech, ctl, alpha_step, alpha_out, status, clin); break;
     case 9:
-      if (g.chem_fixed)
+      if (g.chem_fixed && chem_blocks_per_sm(g.n) == 3)
+        k_chem_lin<9, true, 3><<<blocks, thr, chem_smem(thr), st>>>(S, g, mech, ctl, alpha_step, alpha_out, status, clin);
+      else if (g.chem_fixed)
         k_chem_lin<9, true><<<blocks, thr, chem_smem(thr), st>>>(S, g, mech, ctl, alpha_step, alpha_out, status, clin);
       else
         k_chem_lin<9, false><<<blocks, thr, 0, st>>>(S, g, mech, ctl, alpha_step, alpha_out, status, clin);

@@ -37,6 +37,9 @@ __host__ __device__ constexpr int lines_of(int nv) { return nv == 6 ? 16 : 8; }
 // Blocks an SM is asked to hold: 15 or 16 warps, so 128 registers a thread;
 // 132 would leave room for 12 warps (0.589 ms where 15 take 0.557).
 __host__ __device__ constexpr int blocks_of(int nv) { return 512 / (lines_of(nv) * nv); }
+// With the derivatives 12 warps, so 168 registers (128 spill: 7.02 ms for the
+// adjoint of 1000 x 400 where 168 take 6.73).
+__host__ __device__ constexpr int lin_blocks_of(int nv) { return 384 / (lines_of(nv) * nv); }
 constexpr int FACES = 32;  // faces per tile of the batched launch and of large grids
 
 // One tile of the face-flux launch (FC faces per line); `blk` is the tile's
@@ -155,7 +158,7 @@ __global__ void __launch_bounds__(lines_of(NV) * NV, blocks_of(NV)) k_face_flux(
 // reconstruction with respect to its window differences in `lin` (the
 // discrete adjoint's face-derivative store).
 template <int NV, int FC>
-__global__ void __launch_bounds__(lines_of(NV) * NV) k_face_flux_lin(StateView S, const unsigned long long* __restrict__ alpha,
+__global__ void __launch_bounds__(lines_of(NV) * NV, lin_blocks_of(NV)) k_face_flux_lin(StateView S, const unsigned long long* __restrict__ alpha,
                                                               double* __restrict__ Fx, double* __restrict__ Gy,
                                                               double* __restrict__ lin, GridDev g, int nbx, int ntx_x,
                                                               int ntx_y) {

@@ -93,10 +93,9 @@ JANC_HD long long sar(long long x, int n) {
 JANC_HD u64 mulhi(u64 a, u64 b) {
   return (u64)hi32(a) * hi32(b) + (((u64)hi32(a) * lo32(b)) >> 32) + (((u64)lo32(a) * hi32(b)) >> 32);
 }
-// a^2 / 2^64, at most 3 below the exact quotient. 2 wide products.
+// a^2 / 2^64, at most 1 below the exact quotient. 2 wide products.
 JANC_HD u64 sqhi(u64 a) {
-  const u64 t = ((u64)hi32(a) * lo32(a)) >> 32;
-  return (u64)hi32(a) * hi32(a) + t + t;
+  return (u64)hi32(a) * hi32(a) + (((u64)hi32(a) * lo32(a)) >> 31);
 }
 
 // The float below x (rounded towards zero), as bits. The conversion runs at

@@ -173,3 +173,35 @@ def test_square_root_and_signed_conversion(lib):
         for ai, xi in zip(a.tolist(), x.tolist()):
             want = Q(ai) * Q(2) ** e
             assert abs(Q(xi) - want) <= Q(float(np.spacing(abs(xi)))) / 2
+
+
+def test_scaled_conversion_fixed_exponential_and_floats(lib):
+    """a 2^e rounded to nearest and 0 below the normal range; 2^(a 2^-54) within
+    0.9 units in the last place as exp; floats cut towards zero."""
+    rng = np.random.default_rng(8)
+    a = rng.integers(-2 ** 63 + 1, 2 ** 63 - 1, 4000) >> rng.integers(0, 63, 4000)
+    a = np.concatenate([a, [0, 1, -1, 2 ** 31, 2 ** 32 - 1, 2 ** 32, -2 ** 62, 2 ** 63 - 1]])
+    x = np.zeros(a.size)
+    for e in (0, -1022, -1060, -1085, -1200, 900):
+        lib.wh_scaled(a.size, _ptr(a), e, _ptr(x))
+        for ai, xi in zip(a.tolist(), x.tolist()):
+            want = Q(ai) * Q(2) ** e
+            if abs(want) < Q(2) ** -1022:
+                assert xi == 0.0 or abs(xi) == 2.0 ** -1022
+            else:
+                assert abs(Q(xi) - want) <= Q(float(np.spacing(abs(xi)))) / 2
+    mp = pytest.importorskip("mpmath")
+    mp.mp.prec = 160
+    k = np.concatenate([rng.integers(-2 ** 63, 2 ** 63 - 1, 3000), rng.integers(-2 ** 54, 2 ** 54, 1000),
+                        np.array([0, 1, -1, 2 ** 54, -2 ** 54, 2 ** 54 - 1, 510 * 2 ** 54, -512 * 2 ** 54])])
+    y = np.zeros(k.size)
+    lib.wh_exp2(k.size, _ptr(k), _ptr(y))
+    for ki, yi in zip(k.tolist(), y.tolist()):
+        assert abs(mp.mpf(yi) - mp.mpf(2) ** (mp.mpf(ki) / 2 ** 54)) <= 0.9 * np.spacing(yi)
+    f = np.concatenate([rng.standard_normal(2000) * 10.0 ** rng.uniform(-36, 36, 2000), [1.0, -1.0, 2.0 ** -126, -3.0e38]])
+    g = np.zeros(f.size)
+    lib.wh_float(f.size, _ptr(f), _ptr(g))
+    assert np.all(np.abs(g) <= np.abs(f)) and np.all(np.abs(f - g) < 2.0 ** -23 * np.abs(f)) and np.all(f * g > 0)
+    z = np.array([0.0, -0.0, 1e-39, 5e-324])
+    lib.wh_float(4, _ptr(z), _ptr(g))
+    assert np.all(np.abs(g[:4]) <= 2.0 ** -127)

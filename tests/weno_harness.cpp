@@ -48,6 +48,17 @@ void wh_signed(int n, const long long* a, int e, double* x) {
   for (int i = 0; i < n; ++i) x[i] = soft::signed_double(a[i], e);
 }
 
+// a 2^e as a double, 0 below the normal range; 2^(a 2^-54); x cut to a float and back.
+void wh_scaled(int n, const long long* a, int e, double* x) {
+  for (int i = 0; i < n; ++i) x[i] = soft::scaled_double(a[i], e);
+}
+void wh_exp2(int n, const long long* a, double* x) {
+  for (int i = 0; i < n; ++i) x[i] = soft::exp2_fixed(a[i]);
+}
+void wh_float(int n, const double* x, double* y) {
+  for (int i = 0; i < n; ++i) y[i] = soft::widen(soft::cut_float(x[i]));
+}
+
 // y[i] = 2^127 / (x[i] 2^z[i]) and b[i] = x[i] 2^-64 as a double.
 void wh_soft(int n, const unsigned long long* x, unsigned long long* y, int* z, double* b) {
   for (int i = 0; i < n; ++i) {
