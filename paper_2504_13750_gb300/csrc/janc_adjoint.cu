@@ -1424,21 +1424,32 @@ cudaError_t launch_rhs_vjp(int ns, const StateView& S, const double* alpha2_dev,
   }
 }
 
+// Threads per block of the chemistry VJP: 128 while that gives at least 4 blocks
+// per SM, else 64 or 32, so that all SMs get the same share (512 x 64 in blocks of
+// 128 is 1.7 blocks an SM: 74 us; in blocks of 32: 66 us).
+static int vjp_threads(long long n) {
+  int t = 128;
+  while (t > 32 && (n + t - 1) / t < 4LL * sm_count()) t /= 2;
+  return t;
+}
+
 cudaError_t launch_chem_vjp(int ns, const StateView& Sstar, const GridDev& g, const MechDev* mech, double dt,
                             const double* lam, double* out, const double* clin, cudaStream_t st) {
+  const int thr = vjp_threads(g.n);
+  const unsigned blocks = nblk(g.n, thr);
   if (clin) {
     switch (ns) {
-      case 3: k_adj_chem_lin<3, false><<<nblk(g.n, 128), 128, 0, st>>>(Sstar, g, mech, dt, lam, out, clin); break;
+      case 3: k_adj_chem_lin<3, false><<<blocks, thr, 0, st>>>(Sstar, g, mech, dt, lam, out, clin); break;
       case 9:
-        if (g.chem_fixed) k_adj_chem_lin<9, true><<<nblk(g.n, 128), 128, 0, st>>>(Sstar, g, mech, dt, lam, out, clin);
-        else k_adj_chem_lin<9, false><<<nblk(g.n, 128), 128, 0, st>>>(Sstar, g, mech, dt, lam, out, clin);
+        if (g.chem_fixed) k_adj_chem_lin<9, true><<<blocks, thr, 0, st>>>(Sstar, g, mech, dt, lam, out, clin);
+        else k_adj_chem_lin<9, false><<<blocks, thr, 0, st>>>(Sstar, g, mech, dt, lam, out, clin);
         break;
       default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
   }
   switch (ns) {
-    case 3: k_adj_chem_rev<3, false><<<nblk(g.n, 128), 128, 0, st>>>(Sstar, g, mech, dt, lam, out); break;
+    case 3: k_adj_chem_rev<3, false><<<blocks, thr, 0, st>>>(Sstar, g, mech, dt, lam, out); break;
     case 9:
       if (g.chem_fixed) {
         const int smem = (int)(sizeof(double) * 4 * fixed_h2air::NR * 128);
@@ -1446,9 +1457,9 @@ cudaError_t launch_chem_vjp(int ns, const StateView& Sstar, const GridDev& g, co
         const cudaError_t e = set_attr_once((const void*)k_adj_chem_rev<9, true>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem, &attr_done);
         if (e != cudaSuccess) return e;
-        k_adj_chem_rev<9, true><<<nblk(g.n, 128), 128, smem, st>>>(Sstar, g, mech, dt, lam, out);
+        k_adj_chem_rev<9, true><<<blocks, thr, smem / 128 * thr, st>>>(Sstar, g, mech, dt, lam, out);
       } else {
-        k_adj_chem_rev<9, false><<<nblk(g.n, 128), 128, 0, st>>>(Sstar, g, mech, dt, lam, out);
+        k_adj_chem_rev<9, false><<<blocks, thr, 0, st>>>(Sstar, g, mech, dt, lam, out);
       }
       break;
     default: return cudaErrorInvalidValue;
