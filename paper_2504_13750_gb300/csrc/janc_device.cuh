@@ -496,7 +496,7 @@ __device__ __forceinline__ int newton_cell(const double* u, double Tw, const Mec
   int st = 0;
   int it = 0;
   bool found = false;
-  if (early && maxit >= 4) {
+  if (early && maxit >= 8) {  // so that the iterations would have converged too
     const float f4 = soft::cut_float(h[4]), f3 = soft::cut_float(h[3]), f2 = soft::cut_float(h[2]),
                 f1 = soft::cut_float(h[1]), k1 = soft::cut_float(K1), k0 = soft::cut_float(K0);
     float x = soft::cut_float(Tw);
