@@ -205,3 +205,24 @@ def test_scaled_conversion_fixed_exponential_and_floats(lib):
     z = np.array([0.0, -0.0, 1e-39, 5e-324])
     lib.wh_float(4, _ptr(z), _ptr(g))
     assert np.all(np.abs(g[:4]) <= 2.0 ** -127)
+
+
+@pytest.mark.parametrize("eps", [1e-130, 1e-140, 1e-150, 1e-200, 1e-300])
+def test_derivatives_at_small_epsilon(lib, eps):
+    """Indicators up to 2^2050 apart, where a weight leaves the range of doubles:
+    one, two or three values of a window equal (a flat substencil) beside
+    differences of 1e-3 to 1e10. The bars of test_faces_and_derivatives."""
+    rng = np.random.default_rng(int(-np.log10(eps)))
+    n = 120
+    jump = np.arange(6)[None] >= rng.integers(0, 7, (n, 1))
+    size = 10.0 ** rng.uniform(-3, 10, (n, 6))
+    for F in (jump * size[:, :1], np.where(jump, size, 1e9), size * rng.standard_normal((n, 6))):
+        F = np.ascontiguousarray(F)
+        s, d = _faces(lib, F, F, eps)
+        for i in range(n):
+            f = [Q(float(v)) for v in F[i]]
+            vp, gp = _exact(f[0:5], Q(eps))
+            vm, gm = _exact(f[5:0:-1], Q(eps))
+            assert abs(Q(s[i]) - (vp + vm)) <= 12 * Q(2) ** -53 * max(abs(v) for v in f)
+            for a, b in zip(d[i], gp + [-g for g in gm[::-1]]):
+                assert np.isfinite(a) and abs(Q(float(a)) - b) <= Q(2) ** -44 * max(1, abs(b))
