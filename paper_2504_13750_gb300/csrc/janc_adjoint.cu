@@ -1355,8 +1355,14 @@ static int adj_cell_blocks(const GridDev& g) {
   return ((g.nx + 31) / 32) * ((g.ny + by - 1) / by);
 }
 
+// Doubles of the x faces' per-position sums (pairs): a multiple of 16 bytes.
+static size_t gf_x_doubles(int nv, const GridDev& g) { return 2 * (size_t)nv * g.ny * (g.nx + 6); }
+
+// 24 bytes per 32 x 8 cells, whatever the blocks of the cell pass: callers size
+// workspaces by this number (janc_rhs_vjp). The launch itself uses two doubles of it.
 size_t rhs_vjp_scratch_bytes(const GridDev& g) {
-  return 256 + (((size_t)adj_cell_blocks(g) * 2 * (sizeof(unsigned long long) + sizeof(int)) + 255) & ~(size_t)255);
+  const size_t nb = (size_t)((g.nx + 31) / 32) * ((g.ny + 7) / 8);
+  return 256 + ((24 * nb + 255) & ~(size_t)255);
 }
 
 template <int NS>
@@ -1366,7 +1372,10 @@ static cudaError_t rhs_vjp_t(const StateView& S, const double* alpha2_dev, const
   constexpr int NV = NS + 3, VLINES = vlines_of(NV);
   const int nb = adj_cell_blocks(g);
   double* adj_alpha = scratch;
-  unsigned long long* part_mx = (unsigned long long*)((char*)scratch + 256);
+  // The arg-max partials (3 doubles a block) lie behind the sums in CFx: of its 10 nv
+  // values per face the sums leave nv ny (8 nx - 2), and a block has at least one
+  // row of up to 32 cells, so 24 ny doubles or more are there for 3 ny ceil(nx / 32).
+  unsigned long long* part_mx = (unsigned long long*)(CFx + gf_x_doubles(NV, g));
   int* part_id = (int*)(part_mx + 2 * nb);
   const double* mu = io.lam;
   const double ms = io.mu_scale;
@@ -1374,7 +1383,7 @@ static cudaError_t rhs_vjp_t(const StateView& S, const double* alpha2_dev, const
     // CFx / CFy hold the per-position sums (GF of k_adj_faces); the cell
     // pass and k_adj_alpha leave them and the alpha cotangents zero
     cudaError_t e = cudaMemsetAsync(adj_alpha, 0, 2 * sizeof(double), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(CFx, 0, sizeof(double) * 2 * (size_t)NV * g.ny * (g.nx + 6), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(CFx, 0, sizeof(double) * gf_x_doubles(NV, g), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(CFy, 0, sizeof(double) * 2 * (size_t)NV * (g.ny + 6) * g.nx, st);
     if (e != cudaSuccess) return e;
   }

@@ -89,8 +89,7 @@ bool fixed_structure(const janc_mechanism* m);
 int sm_count();
 
 // Adjoint pieces (janc_adjoint.cu).
-// Scratch of one launch_rhs_vjp: the two alpha cotangents and the per-block
-// arg-max partials of the LF speeds (256-byte aligned start).
+// Scratch of one launch_rhs_vjp (the two alpha cotangents).
 size_t rhs_vjp_scratch_bytes(const GridDev& g);
 // Input and outputs of one RHS vector-Jacobian product nu = (dL/dU)^T mu
 // with mu = mu_scale lam, fused with the linear combinations of an RK stage
@@ -109,6 +108,7 @@ struct VjpIO {
   double cb;
   int acc_b;
 };
+// CFx, CFy: 10 nv doubles per x- and per y-face, 16-byte aligned.
 // lin: the state's face-derivative store (launch_face_flux_lin), or null to
 // recompute the reconstructions. fresh: zero the per-position sums and the
 // alpha cotangents first; otherwise they must be zero on entry (every call

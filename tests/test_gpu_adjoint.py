@@ -605,3 +605,35 @@ def test_run_time_table_chemistry_dot_product(J, store):
         a, b = float(np.sum(seed * dUN[l])), float(np.sum(gU0 * V[l]))
         assert abs(a - b) <= 1e-8 * np.sum(np.abs(seed * dUN[l])), (l, a, b)
     g.close()
+
+
+def _header_bytes(nx, ny, nv):
+    """The workspace of janc_rhs_vjp as include/janc.h states it."""
+    up = lambda b: (b + 255) // 256 * 256  # noqa: E731
+    return (2 * up(8 * nv * nx * ny) + up(80 * nv * ny * (nx + 1)) + up(80 * nv * (ny + 1) * nx)
+            + 256 + up(24 * ((nx + 31) // 32) * ((ny + 7) // 8)))
+
+
+@pytest.mark.parametrize("nx,ny", [(24, 12), (3, 3), (200, 37), (33, 130), (700, 130)])
+def test_rhs_vjp_takes_the_stated_workspace(J, nx, ny):
+    """A workspace of the stated size gives what an internal one gives (bar: the
+    atomic sums of the alpha cotangents come in any order) and nothing behind it
+    is written; 256 bytes less are refused."""
+    import torch
+
+    st, U = _state(nx, ny, 17)
+    nbytes, guard = _header_bytes(nx, ny, U.shape[0]), 1 << 16
+    g = J.Grid.from_grid_dict(H2AIR, st["grid"])
+    g.set_state(U, st["T"])
+    mu = np.random.default_rng(18).normal(size=U.shape)
+    want, nu = np.zeros_like(U), np.zeros_like(U)
+    J.janc_rhs_vjp(g.handle, mu, want)
+    ws = torch.full((nbytes + guard + 256,), 0xA5, dtype=torch.uint8, device="cuda")
+    base = (-ws.data_ptr()) % 256
+    with pytest.raises(J.JancError):
+        J.janc_rhs_vjp(g.handle, mu, nu, ws.data_ptr() + base, nbytes - 256)
+    J.janc_rhs_vjp(g.handle, mu, nu, ws.data_ptr() + base, nbytes)
+    assert bool((ws[base + nbytes:] == 0xA5).all())
+    for k in range(U.shape[0]):
+        assert np.max(np.abs(nu[k] - want[k])) <= 1e-12 * np.max(np.abs(want[k]))
+    g.close()
