@@ -296,8 +296,9 @@ int janc_adjoint_reverse(janc_grid_t g, const double* seed, double* dL_dU0, int 
  * state: nu = (dL/dU)^T mu, both [nv][ny][nx], host or device. workspace:
  * device memory for 2 nv planes plus 10 nv values per x- and y-face, each
  * piece rounded up to 256 bytes, plus 256 bytes and 24 bytes per 32 x 8
- * block of cells rounded up to 256 (NULL: allocated here); a smaller
- * workspace returns JANC_E_NOMEM. Synchronous. */
+ * block of cells rounded up to 256 (NULL: allocated here), 8-byte aligned; a
+ * smaller workspace returns JANC_E_NOMEM, a misaligned one JANC_E_INVALID.
+ * Synchronous. */
 int janc_rhs_vjp(janc_grid_t g, const double* mu, double* nu, void* workspace, size_t workspace_bytes, int where);
 
 /* dL/dT [ny][nx] of the primitive initialisation of Eq. 4.2 at fixed p, u,

@@ -793,6 +793,12 @@ int janc_rhs_vjp(janc_grid_t g, const double* mu, double* nu, void* workspace, s
     own = true;
   } else if (workspace_bytes < need) {
     return fail(JANC_E_NOMEM, "janc_rhs_vjp: workspace too small");
+  } else if ((uintptr_t)ws & 7u) {
+    return fail(JANC_E_INVALID, "janc_rhs_vjp: misaligned workspace");
+  } else {
+    // the pairs of the cell pass are 16-byte accesses; the last piece uses 16 of its
+    // 256 bytes or more, so all of them can move up by 8
+    ws = (char*)(((uintptr_t)ws + 15) & ~(uintptr_t)15);
   }
   double* dmu = (double*)ws;
   double* dnu = (double*)(ws + align256(sizeof(double) * nvn));

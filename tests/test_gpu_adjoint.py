@@ -637,3 +637,31 @@ def test_rhs_vjp_takes_the_stated_workspace(J, nx, ny):
     for k in range(U.shape[0]):
         assert np.max(np.abs(nu[k] - want[k])) <= 1e-12 * np.max(np.abs(want[k]))
     g.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(24, 12), (33, 5), (200, 37)])
+def test_rhs_vjp_takes_workspaces_on_8_byte_boundaries(J, nx, ny):
+    """Workspaces at every multiple of 8 bytes give the result of an internal
+    one (bar as above) and write nothing outside; other addresses are refused."""
+    import torch
+
+    st, U = _state(nx, ny, 19)
+    nbytes = _header_bytes(nx, ny, U.shape[0])
+    g = J.Grid.from_grid_dict(H2AIR, st["grid"])
+    g.set_state(U, st["T"])
+    mu = np.random.default_rng(20).normal(size=U.shape)
+    want = np.zeros_like(U)
+    J.janc_rhs_vjp(g.handle, mu, want)
+    ws = torch.full((nbytes + 1024,), 0xA5, dtype=torch.uint8, device="cuda")
+    base = (-ws.data_ptr()) % 256
+    for off in (4, 12, 257):
+        with pytest.raises(J.JancError):
+            J.janc_rhs_vjp(g.handle, mu, np.zeros_like(U), ws.data_ptr() + base + off, nbytes)
+    for off in (8, 16, 24, 200):
+        ws.fill_(0xA5)
+        nu = np.zeros_like(U)
+        J.janc_rhs_vjp(g.handle, mu, nu, ws.data_ptr() + base + off, nbytes)
+        assert bool((ws[:base + off] == 0xA5).all()) and bool((ws[base + off + nbytes:] == 0xA5).all())
+        for k in range(U.shape[0]):
+            assert np.max(np.abs(nu[k] - want[k])) <= 1e-12 * np.max(np.abs(want[k]))
+    g.close()
