@@ -496,7 +496,9 @@ __device__ __forceinline__ int newton_cell(const double* u, double Tw, const Mec
   int st = 0;
   int it = 0;
   bool found = false;
-  if (early && maxit >= 8) {  // so that the iterations would have converged too
+  // maxit: so that the iterations would have converged too; Tw positive, below 2^100: no
+  // other has a float (NaN or infinity would come out as an ordinary number)
+  if (early && maxit >= 8 && (unsigned)(__double2hiint(Tw) >> 20) - 923u < 200u) {
     const float f4 = soft::cut_float(h[4]), f3 = soft::cut_float(h[3]), f2 = soft::cut_float(h[2]),
                 f1 = soft::cut_float(h[1]), k1 = soft::cut_float(K1), k0 = soft::cut_float(K0);
     float x = soft::cut_float(Tw);
