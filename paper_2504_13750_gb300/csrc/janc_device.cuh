@@ -473,8 +473,10 @@ __device__ __forceinline__ void block_reduce_alpha_status(unsigned long long sx,
 // Three iterations in single precision, then one in double with the second-order
 // term of the root (Chebyshev's iteration; that term only, a 2^-36th of T at
 // most, is formed in single precision), give the same T: accepted where that one
-// step is below 2^-18 T, which leaves a third-order rest below 2^-55 T and the
-// rounding of F, as after any Newton step. 12 FP64 instructions instead of
+// step is below 2^-18 T and s, the term's share of it, below 2^-19. The third-order
+// rest is then below 2^-55 T (2 s^2 of the step, and the third derivative's for heat
+// capacities that vary on the scale of T); the rounding of F remains, as after any
+// Newton step. 12 FP64 instructions instead of
 // three iterations' 33 (of 143 in a stage update of 12 variables: 16.4 us at
 // 512 x 64 then, 14.6 now; one variable's gas at 1021 x 257: 50.9 and 43.5 us). Anything
 // else, so every state that does not converge at once, takes the iterations from
@@ -517,7 +519,7 @@ __device__ __forceinline__ int newton_cell(const double* u, double Tw, const Mec
       const float Fpp = fmaf(x, fmaf(x, fmaf(x, 4.0f * g4, 3.0f * g3), 2.0f * g2), g1);
       const float s = 0.5f * __fdividef(Fpp, soft::cut_float(Fp)) * soft::cut_float(dT);
       // F' within 2^+-100 (positive): its float and the quotient are sound
-      found = dbits(dabs(dT)) + (18ull << 52) <= dbits(y) && fabsf(s) < 0x1p-16f &&
+      found = dbits(dabs(dT)) + (18ull << 52) <= dbits(y) && fabsf(s) < 0x1p-19f &&
               (unsigned)(__double2hiint(Fp) >> 20) - 923u < 200u;
       if (found) t = y + fma(-dT, soft::widen(s), dT);
     }
