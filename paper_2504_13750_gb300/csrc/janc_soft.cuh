@@ -124,12 +124,11 @@ JANC_HD Num normal(u64 x, int e) {
   return Num{shl(x, z), e - z};
 }
 
-// x 2^(e - 64) as a double, truncated to 53 bits, for x >= 2^32; 0 below the
-// normal range. No check against overflow.
+// x 2^(e - 64) as a double, truncated to 53 bits, for x >= 2^32. No range
+// check on the result's exponent.
 JANC_HD double to_double(u64 x, int e) {
   const int z = leading_zeros(hi32(x));
-  const int f = 1021 + e - z;
-  return double_of(f < 0 ? 0ull : (shl(x, z) >> 11) + ((u64)((u32)f << 20) << 32));
+  return double_of((shl(x, z) >> 11) + ((u64)(u32)((1021 + e - z) << 20) << 32));
 }
 
 // 2^127 / d within 8 units for d in [2^63, 2^64), in (2^63, 2^64); fb is the

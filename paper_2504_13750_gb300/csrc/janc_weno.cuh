@@ -174,11 +174,13 @@ struct Coef {
   double k1, k2, k3, k4;
   JANC_HD explicit Coef(const Weights& w) : u0(mulhi(w.u0, w.y)), u1(mulhi(w.u1, w.y)), u2(mulhi(w.u2, w.y)) {
     const u64 v1 = u1 >> 3, v2 = u2 >> 3;
-    const int m = w.d0 < w.d1 ? w.d0 : w.d1, n = w.d1 < w.d2 ? w.d1 : w.d2;
-    k1 = to_double(u0, w.x - 4 - 2 * w.d0);
-    k2 = to_double(3 * shr(v1, 2 * (w.d1 - m)) + 5 * shr(u0, 2 * (w.d0 - m) + 4), w.x - 1 - 2 * m);
-    k3 = to_double(3 * (shr(v1, 2 * (w.d1 - n)) + shr(v2, 2 * (w.d2 - n))), w.x - 2 * n);
-    k4 = to_double(3 * (u2 >> 2), w.x - 3 - 2 * w.d2);
+    // a weight below 2^-960 as one of that size: its exponent stays that of a double
+    const int d0 = w.d0 < 480 ? w.d0 : 480, d1 = w.d1 < 480 ? w.d1 : 480, d2 = w.d2 < 480 ? w.d2 : 480;
+    const int m = d0 < d1 ? d0 : d1, n = d1 < d2 ? d1 : d2;
+    k1 = to_double(u0, w.x - 4 - 2 * d0);
+    k2 = to_double(3 * shr(v1, 2 * (d1 - m)) + 5 * shr(u0, 2 * (d0 - m) + 4), w.x - 1 - 2 * m);
+    k3 = to_double(3 * (shr(v1, 2 * (d1 - n)) + shr(v2, 2 * (d2 - n))), w.x - 2 * n);
+    k4 = to_double(3 * (u2 >> 2), w.x - 3 - 2 * d2);
   }
 };
 
