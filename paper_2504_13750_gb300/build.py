@@ -19,6 +19,8 @@ LIB = os.path.join(BUILD, "libjanc.so")
 SOURCES = ["janc_flux.cu", "janc_update.cu", "janc_chem.cu", "janc_capi.cu", "janc_probe.cu", "janc_static.cu", "janc_server.cu", "janc_adjoint.cu", "janc_amr.cu",
            "janc_slab.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
+# no contraction: the chemistry kernels' variants have to give the same bits
+FLAGS_OF = {"janc_chem.cu": ["-fmad=false"]}
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE]
 
 
@@ -33,7 +35,7 @@ def nvcc() -> str:
 
 
 def _deps():
-    return [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(INCLUDE, "janc.h")]
+    return [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(INCLUDE, "janc.h"), __file__]
 
 
 def up_to_date() -> bool:
@@ -55,7 +57,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
     def compile_one(src):
         obj = os.path.join(BUILD, src.replace(".cu", ".o"))
-        cmd = [cc] + FLAGS + ["-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [cc] + FLAGS + FLAGS_OF.get(src, []) + ["-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stdout}\n{r.stderr}")

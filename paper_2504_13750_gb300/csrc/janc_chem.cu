@@ -18,12 +18,17 @@
 // reaction's species, coefficients and third-body data from the run-time
 // table, FixRx<I> returns them as compile-time constants of the shipped H2-air
 // mechanism (janc_mech_fixed.cuh). From the rate constants on both run the same
-// operations in the same order (the compiler may still contract multiply-adds
-// differently in the two, so their results agree to rounding, each within the
-// oracle's bars); with FixRx the rate constants come from fixed-point logarithms
+// operations in the same order (they agree to rounding, each within the oracle's
+// bars); with FixRx the rate constants come from fixed-point logarithms
 // (rate_constants), and every index of the per-cell arrays (concentrations,
 // production rates, Jacobian) is a constant, so that the arrays live in registers
 // instead of local memory.
+//
+// This file is compiled without contraction (-fmad=false), and the multiply-adds are
+// written as fma: a cell gets the same bits from every kernel below, and which of
+// them a grid takes depends on its size, on its being a slab or a request, and on
+// the adjoint's store. As fast as with the compiler's own contraction (reactors
+// 300 x 101: 72.5 us a step with both, 2048 x 256: 873 us).
 //
 // Bound: 840 FP64 of 12,000 instructions a cell at 8 or 12 warps an SM, the FP64
 // pipe 60 to 70 % busy: that pipe and the length of a cell's chain together.
@@ -91,6 +96,15 @@ __device__ __forceinline__ void rate_constants(const MechDev& m, double T, doubl
   }
 }
 
+// y + nu ab for ab = a b; with the compiled structure, where nu is mostly +-1, one
+// fma and no product (with the rounded product and an addition 300 x 101 takes 76.3 us).
+template <bool FIXED>
+__device__ __forceinline__ double add_times(double nu, double a, double b, double ab, double y) {
+  if (FIXED && nu == 1.0) return fma(a, b, y);
+  if (FIXED && nu == -1.0) return fma(-a, b, y);
+  return fma(nu, ab, y);
+}
+
 // One CHEM_THREADS block `blk` of cells; shared by the single-grid and the
 // batched kernels. STORE (the discrete adjoint's segment recompute): also
 // keep, per cell, what the chemistry VJP reuses (chem_lin_entries doubles,
@@ -133,7 +147,8 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
     X[NSP] = rest * m.invM[NSP];
     double Ctot = X[0];
 #pragma unroll
-    for (int k = 1; k < NS; ++k) Ctot += X[k];
+    for (int k = 1; k < NS; ++k)  // (a sum of X: 1024 x 128 reactors 247 to 256 us; fma with a table: 937 to 963 us, 1024 x 256)
+      Ctot = FIXED ? fma(k < NSP ? u[4 + k] : rest, m.invM[k], Ctot) : Ctot + X[k];
 
     const double lnT = FIXED ? 0.0 : log_t(T);
     const double rT = FIXED ? 0.0 : rcp(T);
@@ -188,6 +203,7 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
       // law of mass action and its derivatives with respect to each
       // participant; a rate is its first derivative times that concentration
       double xr[MAX_SIDE], xp[MAX_SIDE], dq[2 * MAX_SIDE];
+      double lead[2 * MAX_SIDE], tail[2 * MAX_SIDE];  // dq = lead tail
       int dsp[2 * MAX_SIDE];
 #pragma unroll
       for (int r = 0; r < nre; ++r) xr[r] = X[R.rsp(r)];
@@ -196,11 +212,17 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
 #pragma unroll
       for (int r = 0; r < nre; ++r) {
         double d = R.rnu(r) == 1 ? kf : kf * R.rnud(r);
+        lead[r] = d;
+        tail[r] = 1.0;
 #pragma unroll
         for (int s = 0; s < nre; ++s) {
           const int pw = R.rnu(s) - (s == r ? 1 : 0);
 #pragma unroll
-          for (int t = 0; t < pw; ++t) d *= xr[s];
+          for (int t = 0; t < pw; ++t) {
+            lead[r] = d;
+            tail[r] = xr[s];
+            d *= xr[s];
+          }
         }
         dq[r] = d;
         dsp[r] = R.rsp(r);
@@ -208,24 +230,22 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
 #pragma unroll
       for (int r = 0; r < npr; ++r) {
         double d = R.pnu(r) == 1 ? kb : kb * R.pnud(r);
+        lead[nre + r] = -d;
+        tail[nre + r] = 1.0;
 #pragma unroll
         for (int s = 0; s < npr; ++s) {
           const int pw = R.pnu(s) - (s == r ? 1 : 0);
 #pragma unroll
-          for (int t = 0; t < pw; ++t) d *= xp[s];
+          for (int t = 0; t < pw; ++t) {
+            lead[nre + r] = -d;
+            tail[nre + r] = xp[s];
+            d *= xp[s];
+          }
         }
         dq[nre + r] = -d;
         dsp[nre + r] = R.psp(r);
       }
-      double fwd = kf, bwd = kb;
-      if (R.rnu(0) == 1) {
-        fwd = dq[0] * xr[0];
-      } else {
-#pragma unroll
-        for (int r = 0; r < nre; ++r)
-#pragma unroll
-          for (int q = 0; q < R.rnu(r); ++q) fwd *= xr[r];
-      }
+      double net, bwd = kb;
       if (R.pnu(0) == 1) {
         bwd = -dq[nre] * xp[0];
       } else {
@@ -234,26 +254,39 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
 #pragma unroll
           for (int q = 0; q < R.pnu(r); ++q) bwd *= xp[r];
       }
-      const double net = fwd - bwd;
-      double q = net;
+      if (R.rnu(0) == 1) {
+        net = fma(dq[0], xr[0], -bwd);
+      } else {
+        double fwd = kf;
+#pragma unroll
+        for (int r = 0; r < nre; ++r)
+#pragma unroll
+          for (int q = 0; q < R.rnu(r); ++q) fwd *= xr[r];
+        net = __dadd_rn(fwd, -bwd);
+      }
+      double q = net, Mi = 1.0;
       if (R.tb()) {
-        double Mi = Ctot;
+        Mi = Ctot;
 #pragma unroll
         for (int e = 0; e < R.neff(); ++e) Mi = fma(m.effv[i][e], X[R.effsp(e)], Mi);
         q = Mi * net;
 #pragma unroll
-        for (int d = 0; d < nre + npr; ++d) dq[d] *= Mi;
+        for (int d = 0; d < nre + npr; ++d) {
+          lead[d] = dq[d];
+          tail[d] = Mi;
+          dq[d] *= Mi;
+        }
       }
       // sources: wdot_k += nu_ki q
 #pragma unroll
       for (int r = 0; r < nre; ++r) {
         const int k = R.rsp(r);
-        if (k < NSP) wd[k] = fma(-R.rnud(r), q, wd[k]);
+        if (k < NSP) wd[k] = add_times<FIXED>(-R.rnud(r), net, Mi, q, wd[k]);
       }
 #pragma unroll
       for (int r = 0; r < npr; ++r) {
         const int k = R.psp(r);
-        if (k < NSP) wd[k] = fma(R.pnud(r), q, wd[k]);
+        if (k < NSP) wd[k] = add_times<FIXED>(R.pnud(r), net, Mi, q, wd[k]);
       }
       // rows: every carried species with nonzero net coefficient. A third-body
       // coefficient of one in every column goes to S3; one of the last species
@@ -275,7 +308,7 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
           for (int d = 0; d < nre + npr; ++d) {
             const int j = dsp[d];
             if (j < NSP) {
-              J[k][j] = fma(nu, dq[d], J[k][j]);
+              J[k][j] = add_times<FIXED>(nu, lead[d], tail[d], dq[d], J[k][j]);
             } else {
               const double v = nu * dq[d];
 #pragma unroll
@@ -288,7 +321,7 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
 #pragma unroll
               for (int l = 0; l < NSP; ++l) J[k][l] = fma(v, m.ceff[i][l], J[k][l]);
             } else {
-              S3[k] += v;
+              S3[k] = fma(nu, net, S3[k]);
 #pragma unroll
               for (int e = 0; e < R.neff(); ++e) J[k][R.effsp(e)] = fma(v, m.effv[i][e], J[k][R.effsp(e)]);
             }

@@ -490,8 +490,7 @@ __device__ __forceinline__ int newton_cell(const double* u, double Tw, const Mec
   mixture_sums<NS, 6>(u, m, W, h);
   const double c1 = 2.0 * h[1], c2 = 3.0 * h[2], c3 = 4.0 * h[3], c4 = 5.0 * h[4];
   const double ke = fma(u[1], u[1], u[2] * u[2]);
-  const double rhoe_R = fma(-0.5 * rrho, ke, u[3]) * (1.0 / RU);
-  const double K0 = h[5] - rhoe_R;
+  const double K0 = fma(-fma(-0.5 * rrho, ke, u[3]), 1.0 / RU, h[5]);
   const double K1 = h[0] - W;
   const bool early = tol >= 0x1p-50 && tol <= 0x1p-28;
   double t = Tw;
@@ -528,7 +527,7 @@ __device__ __forceinline__ int newton_cell(const double* u, double Tw, const Mec
     double F = fma(t, fma(t, fma(t, fma(t, fma(t, h[4], h[3]), h[2]), h[1]), K1), K0);
     double Fp = fma(t, fma(t, fma(t, fma(t, c4, c3), c2), c1), K1);
     double dT = -F * rcp(Fp);
-    t += dT;
+    t = __dadd_rn(t, dT);
     // the early test on integers: 2^28 |dT| by its exponent field
     const bool done = early && it + 1 < maxit
                           ? dbits(dabs(dT)) + (28ull << 52) <= dbits(dabs(t)) || !finite_bits(dT)

@@ -240,3 +240,16 @@ def test_two_standalone_slabs_in_two_threads(J, bc):
     for p in peers:
         p.close()
     assert np.array_equal(U, Uw) and np.array_equal(T, Tw)
+
+
+@pytest.mark.parametrize("nx,ny,slabs", [(320, 128, 2), (320, 128, 3), (700, 130, 2), (1024, 96, 4)])
+@pytest.mark.parametrize("chem", [1, 2])
+def test_split_across_the_chemistry_kernels(J, nx, ny, slabs, chem):
+    """Domains whose slabs take another variant of the chemistry kernel than the
+    undivided grid (it is chosen by the number of cells): bit for bit all the same.
+    300 to 3500 K, so that every cell reacts."""
+    st = _tube(nx, ny, vel=80.0, seed=3)
+    st["T"] = st["T"] + np.random.default_rng(1).uniform(0.0, 1500.0, st["T"].shape)
+    Uw, Tw, tw = _whole(J, H2AIR, st, chem, 4, cfl=0.5)
+    Us, Ts, ts, _ = _split(J, H2AIR, st, chem, 4, slabs, cfl=0.5)
+    assert np.array_equal(Us, Uw) and np.array_equal(Ts, Tw) and ts == tw
