@@ -50,8 +50,10 @@ constexpr int CHEM_THREADS = 128;
 // dt and the power of P_ref/(Ru T) are summands, so that a reaction takes two
 // exponentials, 2 x 55 integer instructions, and no FP64 one. (As FP64
 // polynomials, nine exp(G_k), their reciprocals and products it was 196 of the
-// cell's 1080 FP64 instructions: 30300 cells in 88 us then, 79 us now.) The logarithms are good to about 2^-51; as
-// doubles, at sizes of 30 to 100, the G_k are good to 2^-48. The sums may wrap on
+// cell's 1080 FP64 instructions: 30300 cells in 88 us then, 79 us with this.) Against 300 bits
+// (H2-air, 257 to 8190 K) the G_k are good to 2^-46.6 and ln k_f to 2^-48.2, where the
+// coefficients' rounding to double, before their conversion, is the limit; as FP64
+// polynomials they were good to 2^-45.9 and 2^-46.1. The sums may wrap on
 // the way, the results are within +-512 (MechDev::rate_ok). Cells outside
 // 256 K <= T < 8192 K, time steps outside 2^-70 .. 2^20 and tables that do not fit
 // take the FP64 form.
@@ -432,12 +434,17 @@ __device__ __forceinline__ void chem_block(const StateView& S, const GridDev& g,
 }
 
 // BLOCKS of the compiled-structure kernels: 3 blocks of 128 threads an SM (12
-// warps) at 168 registers, of which 480 B spill, or no bound (230 registers, 8
+// warps) at 168 registers, of which 516 B spill, or no bound (226 registers, 8
 // warps). A third warp on each scheduler hides more than the spills cost (two steps
 // of 4096 x 512: 20.6 ms with 8, 19.4 with 12), but a full round of 12 takes 86 us
 // where one of 8 takes 74, so the sum of the rounds decides. A step of reactors, us
-// with 8 and with 12: 512 x 96 (10.1 warps an SM) 153 and 112, 512 x 128 (13.5) 154
-// and 153, 640 x 128 (16.8) 223 and 177, 2048 x 256 1033 and 872.
+// with 8 and with 12: 300 x 101 (6.2 warps an SM) 70.3 and 71.3, 512 x 96 (10.1) 150
+// and 109, 512 x 128 (13.5) 153 and 151, 640 x 128 (16.8) 225 and 176, 2048 x 256 1030
+// and 874. With the factors kept (k_chem_lin: 255 registers, 872 B spilled) the same
+// rule; four steps' adjoint forward, ms with 8 and with 12: 512 x 96 2.78 and 2.54,
+// 512 x 128 3.12 and 3.21, 640 x 128 3.86 and 3.81, 700 x 128 4.07 and 4.01, 1024 x 128
+// 5.52 and 5.61 (the one size seen where the rule takes the slower form), 1024 x 256
+// 10.39 and 10.40.
 static int chem_blocks_per_sm(long long n) {
   const long long per = 32LL * sm_count(), w = (n + per - 1) / per;  // warps an SM gets
   return 86 * ((w + 11) / 12) < 74 * ((w + 7) / 8) ? 3 : 0;
@@ -461,7 +468,9 @@ __global__ void __launch_bounds__(CHEM_THREADS, BLOCKS) k_chem_lin(StateView S, 
 }
 
 // Batched chemistry over the flattened (request, block) list: in place on
-// each request's S[0], output alpha in slot 4.
+// each request's S[0], output alpha in slot 4. 12 warps an SM: mixes of many cells gain
+// (24 steps of 369,000 cells 49.9 ms with 8, 48.9 with 12; 167,000: 23.6 and 22.8), of
+// few lose a little (31,000: 5.01 and 5.04; 9,500: 6.50 and 6.58).
 template <int NS, bool FIXED>
 __global__ void __launch_bounds__(CHEM_THREADS, FIXED ? 3 : 0) k_chem_batch(const BatchReq* __restrict__ reqs,
                                                              const int* __restrict__ first, int nreq) {

@@ -1,5 +1,6 @@
 // Device-side data layout and helpers shared by the kernels of the reacting-
-// flow step (arXiv 2504.13750, Sec. 4). All arithmetic is FP64.
+// flow step (arXiv 2504.13750, Sec. 4). State and results are FP64; arithmetic is FP64
+// or 64-bit integer, but for the start of the Newton recovery (newton_cell).
 //
 // GB300 notes that shape this code: the FP64 pipe issues about 2 DFMA per
 // clock per SM (roughly 1/64 of the FP32 rate), while integer, FP32, load and
@@ -78,7 +79,7 @@ struct MechDev {
   unsigned mixs[7][MAX_NS];
   int mixe[7], mixp[MAX_NS];
   int mix_ok;  // every mixe within +-400
-  // G_k and ln k_f as base-2 logarithms in fixed point (fixed_rates): gq in the
+  // G_k and ln k_f as base-2 logarithms in fixed point (fixed_T and below): gq in the
   // order of gc, the factor of log2 T in units of 2^-58, those of (T / 8192)^m and
   // the constant of 2^-54, that of 1/T of 2^-46; kq: ln A, b, -Ea/R likewise;
   // lref = log2(Ru / P_ref) in units of 2^-54. rate_ok: the numbers fit, and every

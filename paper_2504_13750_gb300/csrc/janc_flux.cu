@@ -14,11 +14,13 @@
 // per point instead of once per face, and each thread carries two independent
 // dependency chains.
 //
-// Bound: instruction issue. The FP64 pipe starts one warp instruction every 16
-// clocks, so the nonlinear weights and the weighted sums are formed on the
-// integer pipes (janc_weno.cuh): a face of one variable takes about 800
-// instructions, 8 of them FP64 (67 FP64 when all of it was). 2048 x 256 with 12
-// variables, both directions and their divergence: 1.73 ms then, 0.54 ms now.
+// Bound: instruction issue and the length of the chains (2.6 of 4 instructions a
+// clock, the FP64 pipe 65 % busy). That pipe starts one warp instruction every 16
+// clocks, so the nonlinear weights and the weighted sums are formed on the integer
+// pipes (janc_weno.cuh): a face of one variable takes 780 instructions, 12 of them
+// FP64, the staging and the windows' first values included (67 when all of it was).
+// 2048 x 256 with 12 variables, both directions and their divergence: 1.73 ms then,
+// 0.54 ms now.
 // The loop is not unrolled: by 2 it took 0.59 ms, by 3 0.67 ms (instruction
 // fetch).
 #include <atomic>
@@ -34,8 +36,10 @@ namespace janc {
 // (1000 x 400: 4.68 ms for four steps with 8 lines, 4.07 with 16 and the sums
 // on integers).
 __host__ __device__ constexpr int lines_of(int nv) { return nv == 6 ? 16 : 8; }
-// Blocks an SM is asked to hold: 15 or 16 warps, so 128 registers a thread;
-// 132 would leave room for 12 warps (0.589 ms where 15 take 0.557).
+// Blocks an SM is asked to hold: 15 or 16 warps by registers, 128 a thread; 132
+// would leave room for 12 warps (12 variables: 0.589 ms where 15 take 0.557). Tiles of
+// 32 faces hold fewer by their shared memory for 6 variables (47.4 KB: 4 blocks, 12
+// warps) and for 4 (18.9 KB: 11 of one warp).
 __host__ __device__ constexpr int blocks_of(int nv) { return 512 / (lines_of(nv) * nv); }
 // With the derivatives 12 warps, so 168 registers (128 spill: 7.02 ms for the
 // adjoint of 1000 x 400 where 168 take 6.73).
