@@ -768,46 +768,55 @@ def run_ours(args):
                    "pipeline": "two grids on two streams: one job's host copies beside the other's step; "
                                "the steps one at a time"}
 
-    # ---- the dominant kernel (face fluxes) against the FP64 pipe ----
-    # Most of the operations counted here run as 64-bit integer arithmetic, outside
-    # that pipe, so the shares can exceed one.
-    elsewhere = ("operations of the method as stated over the FP64 pipe's rate; most of them run on the "
-                 "integer pipes (64-bit, at least FP64's accuracy), so the share can exceed 1")
+    # ---- the dominant kernels against the units that bound them ----
+    # Most of the method's operations run as 64-bit integer arithmetic, so its flops
+    # over the FP64 pipe's rate are no roofline; what the kernels execute is: warp
+    # instructions, of which an SM starts 4 a clock, and FP64 ones, of which it
+    # starts one in 16 clocks. Counts per face and variable and per cell from one ncu
+    # capture of these kernels (2048 x 512 tube: 2,099,712 faces, 1,048,576 cells).
     ff_ms, ff_n = prof["face_flux"]
     faces = (nxl + 1) * NY + nxl * (NY + 1)
     flops_launch = nv * faces * (2 * weno_flops() + 1)
     achieved = flops_launch / (ff_ms / ff_n * 1e-3) / 1e12
     peaks = measured_peaks()
-    fp64_nominal = 1.25  # TFLOP/s, GB300 FP64 (recipe's nominal figure)
+    fp64_nominal = 1.25  # TFLOP/s, GB300 FP64, nominal
     dfma = janc.janc_fp64_peak(stream.cuda_stream, 4000)
     fp64_measured = 2.0 * dfma / 1e12
     total_prof = sum(v[0] for v in prof.values())
-    # DRAM bytes per face from one ncu capture of this kernel (2048 x 512 tube,
-    # 12 variables: 248.1 MB read + 172.7 MB written over 2,099,712 faces),
-    # scaled to this launch by its face count.
-    traffic = 420.771e6 / 2099712 * faces if nv == 12 else None
-    roof = {"bound": "alu", "achieved": achieved, "peak": fp64_nominal, "unit": "TFLOP/s",
-            "frac": achieved / fp64_nominal, "traffic": traffic, "kernel": "k_face_flux",
-            "peak_source": "nominal GB300 FP64 1.25 TFLOP/s (152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz)",
-            "peak_measured_dfma_tflops": fp64_measured, "frac_of_measured_dfma": achieved / fp64_measured,
-            "flops_per_launch": flops_launch, "avg_launch_ms": ff_ms / ff_n, "note": elsewhere}
-    # HBM view of the same kernel, beside the FP64 view
+    sms, sm_hz = 152, 2.07e9
+    issue_peak, fp64_issue_peak = 4 * sms * sm_hz / 1e9, sms * sm_hz / 16 / 1e9  # G warp instructions/s
+    ff_s = ff_ms / ff_n * 1e-3
+    issue = 614e6 / (12 * 2099712) * nv * faces / ff_s / 1e9
+    # DRAM bytes of the same capture (248.9 MB read + 176.2 MB written), scaled by the faces
+    traffic = 425.1e6 / 2099712 * faces if nv == 12 else None
+    roof = {"bound": "issue", "achieved": issue, "peak": issue_peak, "unit": "G warp instructions/s",
+            "frac": issue / issue_peak, "traffic": traffic, "kernel": "k_face_flux",
+            "peak_source": "152 SMs x 4 warp instructions/clk x 2.07 GHz",
+            "fp64_pipe_frac": 9.7e6 / (12 * 2099712) * nv * faces / ff_s / 1e9 / fp64_issue_peak,
+            "method": {"flops_per_launch": flops_launch, "tflops": achieved, "over_fp64_nominal": achieved / fp64_nominal,
+                       "fp64_nominal_tflops": fp64_nominal, "measured_dfma_tflops": fp64_measured,
+                       "note": "operations of the method as stated; most run outside the FP64 pipe"},
+            "avg_launch_ms": ff_ms / ff_n}
+    # HBM view of the same kernel
     bytes_launch = 8 * (nv + 2) * cells + 8 * nv * faces  # state + u/v/p planes read, face fluxes written
     hbm = peaks.get("hbm_gbs", 6800.0)
     roof_hbm = {"achieved_gbs": bytes_launch / (ff_ms / ff_n * 1e-3) / 1e9, "peak_gbs": hbm,
                 "frac": bytes_launch / (ff_ms / ff_n * 1e-3) / 1e9 / hbm, "bytes_per_launch": bytes_launch}
     kernels = {k: {"ms_total": v[0], "launches": v[1], "share": v[0] / total_prof if total_prof else None}
                for k, v in prof.items()}
-    # chemistry: FP64 ALU bound; algorithmic flops of the method per cell
+    # chemistry: bound by the FP64 pipe on large grids; algorithmic flops of the method beside it
     ch_ms, ch_n = prof["chemistry"]
+    ch_s = ch_ms / ch_n * 1e-3
     chem_fpc = chem_flops_per_cell(mech)
-    chem_ach = chem_fpc * cells / (ch_ms / ch_n * 1e-3) / 1e12
-    roof_chem = {"bound": "alu", "achieved": chem_ach, "peak": fp64_nominal, "unit": "TFLOP/s",
-                 "frac": chem_ach / fp64_nominal, "kernel": "k_chem", "flops_per_cell": chem_fpc,
-                 "flops_count": "plain analytic form of Eq. 4.6-4.13 and Newton T from the mechanism's structure; "
-                                "FMA = 2 flops, exp/log/reciprocal/sqrt = 1",
-                 "avg_launch_ms": ch_ms / ch_n, "frac_of_measured_dfma": chem_ach / fp64_measured, "note": elsewhere,
-                 "peak_source": "nominal GB300 FP64 1.25 TFLOP/s (152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz)"}
+    chem_ach = chem_fpc * cells / ch_s / 1e12
+    chem_fp64 = 28.1e6 / 1048576 * cells / ch_s / 1e9
+    roof_chem = {"bound": "fp64 pipe", "achieved": chem_fp64, "peak": fp64_issue_peak, "unit": "G FP64 warp instructions/s",
+                 "frac": chem_fp64 / fp64_issue_peak, "kernel": "k_chem",
+                 "peak_source": "152 SMs x 1 FP64 warp instruction per 16 clk x 2.07 GHz",
+                 "method": {"flops_per_cell": chem_fpc, "tflops": chem_ach, "over_fp64_nominal": chem_ach / fp64_nominal,
+                            "flops_count": "plain analytic form of Eq. 4.6-4.13 and Newton T from the mechanism's structure; "
+                                           "FMA = 2 flops, exp/log/reciprocal/sqrt = 1"},
+                 "avg_launch_ms": ch_ms / ch_n}
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True,
